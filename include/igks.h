@@ -75,7 +75,8 @@ typedef struct igks_options {
   int32_t use_graph;      /* capture one iteration (per group) as a CUDA graph and replay it;
                              with 2 <= check_every <= 64 and no timing, also check_every
                              iterations of every group as one graph, launched once per check */
-  int32_t sweep_threads;  /* threads per block of the sweep kernels (0: default) */
+  int32_t sweep_threads;  /* cell threads per block of the sweep kernels, two for each cell of a level
+                             (0: default; at most 256) */
   int32_t timing;         /* record CUDA events around every kernel (igks_kernel_times) */
   int32_t sweep_mode;     /* 0 automatic, 1 one block per solve walking its levels,
                              2 one launch per level over all solves (low-depth orderings) */
@@ -87,11 +88,11 @@ typedef struct igks_options {
                              its own, so that one group's sweeps (one block per solve) overlap
                              another group's flux; same arithmetic, same bits */
   int32_t wait_limit;     /* tries of a device wait (the one-block-per-solve sweeps wait on an
-                             mbarrier for each level's records) before it gives up: the solve
+                             mbarrier for each chunk of records) before it gives up: the solve
                              stops with state IGKS_TIMEOUT, its fields untouched, and
                              igks_iterate returns IGKS_TIMEOUT (0: 2^24 tries, about 1.4 s) */
   int32_t starve_test;    /* test hook, 0 in use: 1 makes every forward sweep skip the copy of
-                             its second level, so that the wait for it runs out */
+                             its second chunk of records, so that the wait for it runs out */
   int32_t reserved[1];
 } igks_options;
 

@@ -53,6 +53,8 @@ struct igks_ctx {
   SolveState* h_st = nullptr;   // pinned mirror of the per-solve state
   int nc_pad = 0, nf = 0, nn = 0;
   std::vector<int> h_wfwd_ptr, h_wbwd_ptr;   // wide schedule level offsets (host copies)
+  std::vector<int> h_pos_b;                  // backward sweep position of every cell (-1 padding)
+  bool ran_wide = false;                     // schedule of the last iterations (igks_get_array)
   // groups of consecutive solves, each iterated on a stream of its own (one group: the
   // context stream); per group its launch ranges, stream, graph and timing events
   int n_groups = 1;
@@ -308,6 +310,7 @@ static int setup_groups(igks_ctx* ctx) {
 // and before whatever the caller puts on it next
 static int run_iterations(igks_ctx* ctx, int n) {
   const int G = ctx->n_groups;
+  if (n > 0) ctx->ran_wide = ctx->dev.wide != 0;
   for (; ctx->bexec && n >= ctx->bgraph_iters; n -= ctx->bgraph_iters)   // whole check intervals
     CK(cudaGraphLaunch(ctx->bexec, ctx->stream));
   if (n == 0) {
@@ -389,6 +392,9 @@ static int build(igks_ctx* ctx) {
   std::vector<int> fs_ptr(1, 0), fs_j, fs_slot, cf_to_fs, bs_ptr(1, 0), bs_j, bs_slot, cf_to_bs;
   std::vector<SolveState> st(ns);
   std::vector<DevFlow> dfl(ns);
+  std::vector<int> gent_ptr(1, 0), gent_pos, fside_ptr, fside_j, bside_ptr, bside_j;
+  const int tbytes = ctx->opt.precision == IGKS_PREC_MIXED ? 4 : 8;
+  const int ring = ring_slots(tbytes), zslot = zero_slot(tbytes);
   for (int s = 0; s < ns; s++) {
     const HostMesh& m = ctx->meshes[s];
     const int co = ctx->cell_off[s], fo = ctx->face_off[s], no = ctx->node_off[s];
@@ -450,7 +456,7 @@ static int build(igks_ctx* ctx) {
     blsp[s + 1] = (int)bwd_lvl.size();
     // narrow-schedule stencils in sweep-position order, with shared-memory ring slots: a
     // neighbour produced at position q is still in the ring while the current level (end
-    // e) is processed iff q >= e - RING (no position written during the level maps to its
+    // e) is processed iff q >= e - ring (no position written during the level maps to its
     // slot)
     cf_to_fs.resize(cf_face.size(), -1);
     cf_to_bs.resize(cf_face.size(), -1);
@@ -464,8 +470,12 @@ static int build(igks_ctx* ctx) {
       std::vector<int>& sj = fwd ? fs_j : bs_j;
       std::vector<int>& sslot = fwd ? fs_slot : bs_slot;
       std::vector<int>& map = fwd ? cf_to_fs : cf_to_bs;
+      std::vector<int>& side_ptr = fwd ? fside_ptr : bside_ptr;
+      std::vector<int>& side_j = fwd ? fside_j : bside_j;
+      const size_t side_max = side_j.size() + m.nc / 4;   // within the solve's footprint bound
       for (int l = 0; l + 1 < (int)lvll.size(); l++) {
         const int e = lvll[l + 1];
+        side_ptr.push_back((int)side_j.size());
         for (int p = lvll[l]; p < e; p++) {
           const int i = ordl[p];
           for (int k = lp[i]; k < lp[i + 1]; k++) {
@@ -477,7 +487,7 @@ static int build(igks_ctx* ctx) {
                            m.face_bc[f] == IGKS_BC_MOVING_WALL)) {
                 map[kg] = (int)sj.size();
                 sj.push_back(-1 - (fo + f));
-                sslot.push_back(-1);
+                sslot.push_back(SLOT_GHOST);
               }
               continue;
             }
@@ -485,11 +495,21 @@ static int build(igks_ctx* ctx) {
             if (fwd ? (j >= i) : (j <= i)) continue;
             map[kg] = (int)sj.size();
             sj.push_back(co + j);
-            sslot.push_back(pos[j] >= e - RING ? pos[j] % RING : -1);
+            // a neighbour that left the ring: its increments are fetched into one of the
+            // level's side slots, from two levels ahead on (they are in global memory by then)
+            int slot = SLOT_GLOBAL;
+            if (pos[j] >= e - ring) slot = pos[j] % ring;
+            else if ((int)side_j.size() - side_ptr.back() < SIDE && side_j.size() < side_max && l >= 3 &&
+                     pos[j] < lvll[l - 2]) {
+              slot = ring + (l & 1) * SIDE + (int)side_j.size() - side_ptr.back();
+              side_j.push_back(co + j);
+            }
+            sslot.push_back(slot);
           }
           sptr.push_back((int)sj.size());
         }
       }
+      side_ptr.push_back((int)side_j.size());
     }
     // state
     SolveState& q = st[s];
@@ -504,18 +524,18 @@ static int build(igks_ctx* ctx) {
   // ---- narrow schedule: per-position padded stencils (PF_E entries) and positions ----
   const int P = (int)fwd_order.size();
   std::vector<int> pos_f(nc, -1), pos_b(nc, -1);
-  std::vector<FwdStat> fst(P);
-  std::vector<BwdStat> bst(P);
+  std::vector<SweepStat> fst(P), bst(P);
+  std::vector<SweepJ> fj(P), bj(P);
   std::vector<int> cf_to_ef(cf_face.size(), -1), cf_to_eb(cf_face.size(), -1);
   for (int p = 0; p < P; p++) { pos_f[fwd_order[p]] = p; pos_b[bwd_order[p]] = p; }
   for (int p = 0; p < P; p++) {
-    FwdStat& f = fst[p];
-    BwdStat& b = bst[p];
-    std::memset(&f, 0, sizeof f);
-    std::memset(&b, 0, sizeof b);
-    f.i = fwd_order[p]; f.pb = pos_b[fwd_order[p]];
-    b.i = bwd_order[p];
-    for (int e = 0; e < PF_E; e++) { f.slot[e] = -1; b.slot[e] = -1; }
+    std::memset(&fst[p], 0, sizeof fst[p]);
+    std::memset(&bst[p], 0, sizeof bst[p]);
+    std::memset(&fj[p], 0, sizeof fj[p]);
+    std::memset(&bj[p], 0, sizeof bj[p]);
+    fst[p].i = fwd_order[p]; fst[p].pb = pos_b[fwd_order[p]];
+    bst[p].i = bwd_order[p];
+    for (int e = 0; e < PF_E; e++) fst[p].slot[e] = bst[p].slot[e] = zslot;
   }
   for (int dir = 0; dir < 2; dir++) {
     const bool fwd = dir == 0;
@@ -523,24 +543,40 @@ static int build(igks_ctx* ctx) {
     const std::vector<int>& sj = fwd ? fs_j : bs_j;
     const std::vector<int>& sslot = fwd ? fs_slot : bs_slot;
     const std::vector<int>& map = fwd ? cf_to_fs : cf_to_bs;
+    const std::vector<int>& pos = fwd ? pos_f : pos_b;
+    std::vector<SweepStat>& rec = fwd ? fst : bst;
     std::vector<int>& emap = fwd ? cf_to_ef : cf_to_eb;
+    std::vector<SweepJ>& recj = fwd ? fj : bj;
     std::vector<int> inv(sj.size(), -1);
     for (size_t k = 0; k < map.size(); k++)
       if (map[k] >= 0) inv[map[k]] = (int)k;
+    for (size_t k = 0; k < sj.size(); k++)   // cells whose increments are read from global memory
+      if (sslot[k] == SLOT_GLOBAL || sslot[k] >= ring) rec[pos[sj[k]]].spill = 1;
     for (int p = 0; p < P; p++) {
-      int* cnt = fwd ? &fst[p].cnt : &bst[p].cnt;
-      int* ej = fwd ? fst[p].j : bst[p].j;
-      int* es = fwd ? fst[p].slot : bst[p].slot;
-      const int q0 = sptr[p], m_ = sptr[p + 1] - q0;
-      if (m_ > PF_E) { *cnt = -1; continue; }
-      *cnt = m_;
+      SweepStat& q = rec[p];
+      int q0 = sptr[p];
+      while (q0 < sptr[p + 1] && sslot[q0] == SLOT_GHOST) q0++;   // ghosts that come first: the sum's start
+      const int m_ = sptr[p + 1] - q0;
+      if (m_ > PF_E) { q.kind = KIND_RARE | KIND_CSR; continue; }
+      q.kind = m_ | (m_ > 2 ? KIND_RARE : 0);
       for (int e = 0; e < m_; e++) {
-        ej[e] = sj[q0 + e];
-        es[e] = sslot[q0 + e];
+        if (sslot[q0 + e] < 0) q.kind |= KIND_RARE;
+        if (sslot[q0 + e] >= ring) q.kind |= KIND_SIDE;
+        recj[p].j[e] = sj[q0 + e];
+        q.slot[e] = sslot[q0 + e];
         emap[inv[q0 + e]] = p * PF_E + e;
       }
     }
   }
+  for (int s = 0, p = 0; s < ns; s++) {      // cells with ghosts in their backward records, per solve
+    for (const int end = p + ctx->meshes[s].nc; p < end; p++) {
+      bool ghost = false;
+      for (int k = bs_ptr[p]; k < bs_ptr[p + 1]; k++) ghost |= bs_slot[k] == SLOT_GHOST;
+      if (ghost && !(bst[p].kind & KIND_CSR)) gent_pos.push_back(p);
+    }
+    gent_ptr.push_back((int)gent_pos.size());
+  }
+  ctx->h_pos_b = pos_b;
   // ---- device buffers ----
   Dev& d = ctx->dev;
   d = Dev{};
@@ -580,10 +616,17 @@ static int build(igks_ctx* ctx) {
   d.nbs = (int)bs_j.size();
   AL(sc_f, double, 4 * (size_t)std::max(d.nfs, 1)); AL(sc_b, double, 4 * (size_t)std::max(d.nbs, 1));
   d.npos = P;
-  UP(pos_f, pos_f); UP(pos_b, pos_b); UP(fst, fst); UP(bst, bst);
+  UP(pos_f, pos_f); UP(pos_b, pos_b);
   UP(cf_to_ef, cf_to_ef); UP(cf_to_eb, cf_to_eb);
-  // per-iteration records, sized for the widest sweep type
-  AL(fdyn, FwdDyn<double>, (size_t)P); AL(bdyn, BwdDyn<double>, (size_t)P);
+  // records, sized for the widest sweep type; their static parts
+  AL(frec, SweepRec<double>, (size_t)P); AL(brec, SweepRec<double>, (size_t)P);
+  const size_t rec = ctx->opt.precision == IGKS_PREC_MIXED ? sizeof(SweepRec<float>) : sizeof(SweepRec<double>);
+  CK(h2d_2d(ctx, d.frec, rec, fst.data(), sizeof(SweepStat), sizeof(SweepStat), P));
+  CK(h2d_2d(ctx, d.brec, rec, bst.data(), sizeof(SweepStat), sizeof(SweepStat), P));
+  UP(fj, fj); UP(bj, bj);
+  UP(fside_ptr, fside_ptr); UP(fside_j, fside_j); UP(bside_ptr, bside_ptr); UP(bside_j, bside_j);
+  UP(gent_ptr, gent_ptr); UP(gent_pos, gent_pos);
+  d.ring = ring;
   AL(gprim, double, 6 * (size_t)nf);
   setup_sweeps();
   {
@@ -894,6 +937,31 @@ static int get_faces(igks_ctx* ctx, int solve, const double* base, int k, double
   return 0;
 }
 
+// the forward increments of the narrow sweeps: the m of the solve's backward records
+static int get_dwstar(igks_ctx* ctx, int solve, double* out) {
+  const int n = ctx->meshes[solve].nc, prec = ctx->opt.precision;
+  const size_t rec = prec == IGKS_PREC_MIXED ? sizeof(SweepRec<float>) : sizeof(SweepRec<double>);
+  const size_t w = prec == IGKS_PREC_MIXED ? 4 : 8;
+  int p0 = 0;
+  for (int s = 0; s < solve; s++) p0 += ctx->meshes[s].nc;
+  std::vector<unsigned char> tmp(5 * w * (size_t)n);
+  CK(d2h_2d(ctx, tmp.data(), 5 * w, (const unsigned char*)ctx->dev.brec + rec * (size_t)p0 + sizeof(SweepStat), rec, 5 * w, n));
+  for (int i = 0; i < n; i++) {
+    const unsigned char* q = tmp.data() + 5 * w * (size_t)(ctx->h_pos_b[ctx->cell_off[solve] + i] - p0);
+    for (int v = 0; v < 5; v++) {
+      double x;
+      if (prec == IGKS_PREC_FP64) std::memcpy(&x, q + 8 * v, 8);
+      else {
+        float f[2] = {0.0f, 0.0f};
+        std::memcpy(f, q + w * v, w);
+        x = (double)f[0] + (double)f[1];
+      }
+      out[(size_t)v * n + i] = x;
+    }
+  }
+  return 0;
+}
+
 int igks_get_fields(igks_ctx* ctx, int32_t solve, double* W) {
   if (check_solve(ctx, solve) || !W) return IGKS_EINVAL;
   int rc = build(ctx);
@@ -1010,6 +1078,7 @@ int igks_get_array(igks_ctx* ctx, int32_t solve, int32_t which, double* out) {
     }
     case IGKS_ARR_DWSTAR:
     case IGKS_ARR_DW: {
+      if (which == IGKS_ARR_DWSTAR && !ctx->ran_wide) return get_dwstar(ctx, solve, out);
       const void* src = which == IGKS_ARR_DWSTAR ? d.dWs : d.dW;
       if (ctx->opt.precision == IGKS_PREC_MIXED) {
         std::vector<float> tmp(5 * (size_t)n);

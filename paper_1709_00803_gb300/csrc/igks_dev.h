@@ -31,37 +31,42 @@ struct DevFlow {
 };
 
 // per-solve iteration state, updated only on the device during iterations
-constexpr int PF_E = 4;              // stencil entries held per sweep record
+constexpr int PF_E = 3;              // stencil entries held per sweep record
 
-// static part of a narrow-sweep record: cell, entry count (-1: CSR stencil), the cell's
-// backward position, and the entries' neighbours (j < 0: wall / symmetry ghost of face
-// -1 - j) and shared-memory ring slots (-1: read from global memory)
-struct alignas(16) FwdStat { int i, cnt, pb, pad; int j[PF_E], slot[PF_E]; };
-struct alignas(16) BwdStat { int i, cnt, pad0, pad1; int j[PF_E], slot[PF_E]; };
-// per-iteration part (T = double, float or double-float): forward: residual M[5], state
-// (r, mx, my), 1/D, 1/a_ii, u, v, H and per entry (sx, sy, s lambda, SA coefficient);
-// backward: state W[5], the same five constants, the forward increment dW*[5], entries.
-// The head (up to the entries) and each entry's four coefficients are whole 16-byte
-// chunks, so the pre-pass writes them with vector stores; every record is an odd number
-// of chunks, so a warp reading its lanes' records from shared memory with 16-byte loads
-// hits distinct banks.
+// Records of the narrow sweeps, one per sweep position and direction, brought into shared
+// memory by bulk copies.
+// Static part (uploaded once): cell, kind (entry count, and the flags below), the cell's
+// backward position (forward records), whether a later cell reads this cell's increments
+// from global memory, and per entry where the neighbour's increments are: a slot of the
+// shared-memory ring, from ring_slots on a side slot (a neighbour that left the ring,
+// fetched again ahead of its level), ZERO_SLOT (no entry: reads zeros, and its coefficients
+// stay zero), SLOT_GLOBAL (read from global memory) or SLOT_GHOST (a wall or symmetry ghost
+// after an interior neighbour, whose mean-flow terms the forward sweep leaves in the entry's
+// coefficients).
+// Per iteration (T = double, float or double-float): m = residual M (forward) or forward
+// increment dW* (backward), state (r, mx, my), 1/D, 1/a_ii, u, v, H, per entry (sx, sy,
+// s lambda, SA coefficient), and the backward sum's start (the ghosts that come first;
+// start[4] in pad0[0]). The static part, the head (m to pad0) and two entries (8-byte types:
+// one) are whole 32-byte sectors, so the pre-pass leaves few sectors partly written (with
+// 176-byte records it took 377 us on a batch of 623,000 cells, with these 135 us), and four
+// consecutive records start on distinct 32-byte bank groups.
+constexpr int SLOT_GLOBAL = -1, SLOT_GHOST = -2;
+constexpr int KIND_COUNT = 7;        // entries
+constexpr int KIND_RARE = 16;        // more than two entries, a ghost, or a neighbour in global memory
+constexpr int KIND_SIDE = 32;        // a side slot (used by staged solves only)
+constexpr int KIND_CSR = 64;         // more than PF_E entries: the CSR stencil (KIND_RARE too)
+struct alignas(16) SweepStat { int i, kind, pb, spill; int slot[PF_E], pad; };
+struct alignas(16) SweepJ { int j[PF_E], pad; };            // the entries' cells, -1 - face for a ghost
 template <class T>
-struct alignas(16) FwdDyn {
+struct alignas(16) SweepRec {
+  SweepStat st;
   T m[5], w[3], c[5];
-  T pad0[sizeof(T) == 4 ? 3 : 1];
+  T pad0[3];
   T co[PF_E][4];
-  T pad1[4];
+  T start[4];
 };
-template <class T>
-struct alignas(16) BwdDyn {
-  T w[5], c[5], ws[5];
-  T pad0[1];
-  T co[PF_E][4];
-  T pad1[sizeof(T) == 4 ? 4 : 2];
-};
-static_assert(sizeof(FwdStat) == 48 && sizeof(BwdStat) == 48, "static record size");
-static_assert(sizeof(FwdDyn<float>) == 144 && sizeof(FwdDyn<double>) == 272, "forward record size");
-static_assert(sizeof(BwdDyn<float>) == 144 && sizeof(BwdDyn<double>) == 272, "backward record size");
+static_assert(sizeof(SweepStat) == 32 && sizeof(SweepJ) == 16, "static record size");
+static_assert(sizeof(SweepRec<float>) == 160 && sizeof(SweepRec<double>) == 288, "record size");
 
 struct SolveState {
   double dt, cfl, res_inf, res_l2, res_l2_first, res_inf_prev, eq40;
@@ -134,18 +139,23 @@ struct Dev {
   void* sc_f; void* sc_b;        // [4][entries] coefficients (T), written by the pre-pass
   int nfs, nbs;                  // entry counts
   // narrow schedule, per sweep position p (P = npos = all real cells): one record per
-  // position and direction, array-of-structures so that a level's records are one
+  // position and direction, array-of-structures so that consecutive records are one
   // contiguous range (one bulk copy); the static part (cell, entry count, neighbours,
   // ring slots) is uploaded once, the per-iteration part written by the pre-pass. Up to
   // PF_E stencil entries per record (cnt < 0: more than that, use the CSR stencil above).
   int npos;
   const int* pos_f; const int* pos_b;            // [nc_pad] position of a cell (-1 padding)
-  const FwdStat* fst; const BwdStat* bst;        // [P]
-  void* fdyn; void* bdyn;                        // [P] FwdDyn<T> / BwdDyn<T>
+  const SweepJ* fj; const SweepJ* bj;            // [P]
+  void* frec; void* brec;                        // [P] SweepRec<T>
+  const int* fside_ptr; const int* bside_ptr;    // per level (indexed as fwd_lvl / bwd_lvl): the cells
+  const int* fside_j; const int* bside_j;        // whose increments go to the level's side slots
+  const int* gent_ptr;                           // [n_solves+1] cells with wall or symmetry ghosts
+  const int* gent_pos;                           // their backward positions (records, not CSR stencils)
+  int ring;                                      // slots of the shared-memory ring
   void* gprim;                                   // [6][nf] T: ghost r, mx, my, u, v, H of wall/symmetry faces
-  const int* cf_to_ef; const int* cf_to_eb;      // [nnz] p * PF_E + e, or -1
+  const int* cf_to_ef; const int* cf_to_eb;      // [nnz] p * PF_E + e, or -1 (not an entry)
   int wait_limit;                // spins of a device wait before it gives up (IGKS_TIMEOUT)
-  int starve_test;               // test hook: the forward sweep never stages its second level
+  int starve_test;               // test hook: the forward sweep never stages its second chunk of records
   int* tmo;                      // [n_solves] a sweep wait of the solve ran out this iteration
   // wide schedule: cells of each level of all solves
   int wide;                      // 1: one launch per level; 0: one block per solve
@@ -192,8 +202,12 @@ void launch_end_iter(const Dev& d, cudaStream_t s);
 // solves that pass into W
 void launch_set_state(const Dev& d, const double* staged, int* bad, cudaStream_t s);
 constexpr int N_KERNEL_KINDS = 11;   // kernels of one iteration (the wide sweeps launch per level)
-constexpr int RING = 1024;           // shared-memory ring of the narrow sweeps (cells)
-constexpr int NARROW_THREADS = 256;  // block of the narrow sweeps (one thread per cell of a level)
+// shared-memory ring of the narrow sweeps (cells) for a sweep type of t bytes: 13 values a
+// cell, 104 KiB either way (a power of two: any cluster size divides it)
+constexpr int ring_slots(int t) { return t == 4 ? 2048 : 1024; }
+constexpr int SIDE = 32;             // side slots of a level (two sets, by the level's parity)
+constexpr int zero_slot(int t) { return ring_slots(t) + 2 * SIDE; }
+constexpr int NARROW_THREADS = 256;  // cell threads of the narrow sweeps (two per cell of a level)
 constexpr int DEFAULT_WAIT_LIMIT = 1 << 24;   // spins of a device wait (about a second)
 constexpr int MAX_BATCH_GRAPH_ITERS = 64;     // iterations captured in one whole-batch graph at most
 constexpr int WIDE_MAX_LEVELS = 64;  // automatic choice: wide schedule up to this many levels

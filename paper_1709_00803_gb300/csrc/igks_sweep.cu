@@ -13,19 +13,18 @@
 //
 // Two schedules:
 //  - narrow: one block per solve (or a thread-block cluster) walks its levels with a
-//    barrier between them (for orderings with hundreds of thin levels). The increments of
-//    the last RING cells it produced stay in a shared-memory ring, so a cell usually reads
-//    its neighbours' increments from shared memory; its record (stencil neighbours, ring
-//    slots, coefficients and per-cell constants) is stored in sweep-position order, and a
-//    level's records are brought into shared memory by bulk copies on an mbarrier, a few
-//    levels ahead;
+//    barrier between them (for orderings with hundreds of thin levels). Two threads work on
+//    a cell; the increments of the last cells it produced stay in a shared-memory ring, so
+//    a cell usually reads its neighbours' increments from shared memory; its record (stencil
+//    neighbours, ring slots, coefficients and per-cell constants) is stored in
+//    sweep-position order, and records are brought into shared memory by bulk copies on
+//    mbarriers several levels ahead, and into registers one level ahead;
 //  - wide: one launch per level covering that level's cells of every solve (for low-depth
 //    orderings, e.g. multicolour, whose few levels hold thousands of cells each).
 #include <cooperative_groups.h>
 #include <float.h>
 
 #include <cstddef>
-
 #include <type_traits>
 
 #include "igks_df64.cuh"
@@ -44,15 +43,16 @@ namespace igks {
 __device__ __forceinline__ double fma_x(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ double mul_x(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double add_x(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double div_x(double a, double b) { return __ddiv_rn(a, b); }
 __device__ __forceinline__ float fma_x(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ float mul_x(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float add_x(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float div_x(float a, float b) { return __fdiv_rn(a, b); }
 __device__ __forceinline__ df64 fma_x(df64 a, df64 b, df64 c) { return a * b + c; }
 __device__ __forceinline__ df64 mul_x(df64 a, df64 b) { return a * b; }
 __device__ __forceinline__ df64 add_x(df64 a, df64 b) { return a + b; }
-__device__ __forceinline__ df64 div_x(df64 a, df64 b) { return a / b; }
+// 1 / x, correctly rounded (the bits of the division in FP64 and FP32, fewer instructions)
+__device__ __forceinline__ double rcp_x(double x) { return __drcp_rn(x); }
+__device__ __forceinline__ float rcp_x(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ df64 rcp_x(df64 x) { return df64(1.0f, 0.0f) / x; }
 
 // Increment of the x and y Euler fluxes for the increment (dr, dmx, dmy, dE) of a state
 // with density r, momenta mx, my, velocity u, v and total enthalpy density H = E + p,
@@ -61,7 +61,7 @@ __device__ __forceinline__ df64 div_x(df64 a, df64 b) { return a / b; }
 template <class T>
 __device__ __forceinline__ void delta_flux(T r, T mx, T my, T u, T v, T H, T dr, T dmx, T dmy, T dE, T* o) {
   const T g1 = (T)(GAMMA - 1.0);
-  const T inv1 = div_x((T)1, add_x(r, dr));
+  const T inv1 = rcp_x(add_x(r, dr));
   const T du = mul_x(fma_x(-u, dr, dmx), inv1);          // (dmx - u dr) / (r + dr)
   const T dv = mul_x(fma_x(-v, dr, dmy), inv1);
   const T u1 = add_x(u, du), v1 = add_x(v, dv);
@@ -99,6 +99,18 @@ __device__ __forceinline__ void fwd_comp(T& a, T sx, T sy, T sl, T f0, T f1, T w
 template <class T>
 __device__ __forceinline__ void bwd_comp(T& a, T sx, T sy, T sl, T f0, T f1, T w) {
   a = add_x(a, entry_sum(sx, sy, sl, f0, f1, w));
+}
+// FP64: three fused multiply-adds onto the accumulator (a warp-wide FP64 instruction costs
+// an SM 19 cycles whatever its active lanes: three instead of four per entry and component)
+template <>
+__device__ __forceinline__ void fwd_comp<double>(double& a, double sx, double sy, double sl, double f0, double f1,
+                                                 double w) {
+  a = fma_x(-sx, f0, fma_x(-sy, f1, fma_x(sl, w, a)));
+}
+template <>
+__device__ __forceinline__ void bwd_comp<double>(double& a, double sx, double sy, double sl, double f0, double f1,
+                                                 double w) {
+  a = fma_x(sx, f0, fma_x(sy, f1, fma_x(-sl, w, a)));
 }
 template <class T>
 __device__ __forceinline__ void fwd_sa(T& a, T sa, T w) { a = fma_x(-sa, w, a); }
@@ -173,6 +185,14 @@ __device__ __forceinline__ void fwd_sa<df64>(df64& a, df64 sa, df64 w) { df_mac(
 template <>
 __device__ __forceinline__ void bwd_sa<df64>(df64& a, df64 sa, df64 w) { df_mac(a, sa, w); }
 
+// The four mean-flow terms of a wall or symmetry ghost are formed ahead of the backward
+// sweep's dependency chain (they need the cell's own forward increment only) and added at
+// the entry's place in the order.
+template <class T>
+__device__ __forceinline__ void ghost_add(T& a, T term) { a = add_x(a, term); }
+template <>
+__device__ __forceinline__ void ghost_add<df64>(df64& a, df64 term) { df_mac(a, df64(1.0f, 0.0f), term); }
+
 // the first BYTES bytes of src to dst (both 16-byte aligned) as 16-byte stores
 template <size_t BYTES>
 __device__ __forceinline__ void store_chunks(void* dst, const void* src) {
@@ -210,25 +230,21 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_sweep_prep(Dev d) {
     for (int q = 0; q < 5; q++) c[q * n + i] = cc[q];
   }
   // position-ordered records of the narrow schedule: the heads as whole 16-byte chunks
-  // (the backward head's dW* slots are written by the forward sweep afterwards)
+  // (the backward head's dW* is written by the forward sweep afterwards)
   const int pf = d.pos_f[i], pb = d.pos_b[i];
-  FwdDyn<T>* rf = (FwdDyn<T>*)d.fdyn + pf;
-  BwdDyn<T>* rb = (BwdDyn<T>*)d.bdyn + pb;
-  const bool csr_f = d.fst[pf].cnt < 0, csr_b = d.bst[pb].cnt < 0;   // more entries than a record holds
+  SweepRec<T>* rf = (SweepRec<T>*)d.frec + pf;
+  SweepRec<T>* rb = (SweepRec<T>*)d.brec + pb;
   if (!wide) {
-    FwdDyn<T> hf;
-    BwdDyn<T> hb;
+    constexpr size_t HEAD = offsetof(SweepRec<T>, co) - offsetof(SweepRec<T>, m);
+    SweepRec<T> h;
+    h.w[0] = (T)r; h.w[1] = (T)mx; h.w[2] = (T)my;
 #pragma unroll
-    for (int q = 0; q < 5; q++) hf.m[q] = (T)d.M[q * n + i];
-    hf.w[0] = (T)r; hf.w[1] = (T)mx; hf.w[2] = (T)my;
+    for (int q = 0; q < 5; q++) { h.c[q] = cc[q]; h.m[q] = (T)0; }
+    for (int q = 0; q < (int)(sizeof(h.pad0) / sizeof(T)); q++) h.pad0[q] = (T)0;
+    store_chunks<HEAD>(rb->m, h.m);
 #pragma unroll
-    for (int q = 0; q < 5; q++) { hf.c[q] = cc[q]; hb.c[q] = cc[q]; hb.ws[q] = (T)0; }
-#pragma unroll
-    for (int q = 0; q < 5; q++) hb.w[q] = (T)d.W[q * n + i];
-    for (int q = 0; q < (int)(sizeof(hf.pad0) / sizeof(T)); q++) hf.pad0[q] = (T)0;
-    hb.pad0[0] = (T)0;
-    store_chunks<offsetof(FwdDyn<T>, co)>(rf, &hf);
-    store_chunks<offsetof(BwdDyn<T>, co)>(rb, &hb);
+    for (int q = 0; q < 5; q++) h.m[q] = (T)d.M[q * n + i];
+    store_chunks<HEAD>(rf->m, h.m);
   }
   T* sc = (T*)d.sw_st;
   const int nnz = d.nnz;
@@ -244,21 +260,21 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_sweep_prep(Dev d) {
       d.sw_j[k] = j;                                  // -1 on a boundary face
       sc[k] = e0; sc[nnz + k] = e1; sc[2 * nnz + k] = e2; sc[3 * nnz + k] = e3;
     } else {
-      // the narrow schedule: up to PF_E entries per position in its record, the rest of a
-      // larger stencil in the position-ordered CSR lists
+      // the narrow schedule: up to PF_E entries per position in its record; a larger stencil
+      // and the ghosts in the position-ordered CSR lists
       const int ef = d.cf_to_fs[k], eb = d.cf_to_bs[k];
-      if (ef >= 0 && csr_f) {
+      const int xf = d.cf_to_ef[k], xb = d.cf_to_eb[k];   // record entry: position * PF_E + e
+      if (ef >= 0 && xf < 0) {
         T* o = (T*)d.sc_f;
         o[ef] = e0; o[d.nfs + ef] = e1; o[2 * d.nfs + ef] = e2; o[3 * d.nfs + ef] = e3;
       }
-      if (eb >= 0 && csr_b) {
+      if (eb >= 0 && (xb < 0 || j < 0)) {
         T* o = (T*)d.sc_b;
         o[eb] = e0; o[d.nbs + eb] = e1; o[2 * d.nbs + eb] = e2; o[3 * d.nbs + eb] = e3;
       }
-      const int xf = d.cf_to_ef[k], xb = d.cf_to_eb[k];   // record entry: position * PF_E + e
       alignas(16) const T ent[4] = {e0, e1, e2, e3};      // one entry: whole 16-byte chunks
-      if (xf >= 0) store_chunks<sizeof(ent)>(((FwdDyn<T>*)d.fdyn)[xf / PF_E].co[xf % PF_E], ent);
-      if (xb >= 0) store_chunks<sizeof(ent)>(((BwdDyn<T>*)d.bdyn)[xb / PF_E].co[xb % PF_E], ent);
+      if (xf >= 0) store_chunks<sizeof(ent)>(((SweepRec<T>*)d.frec)[xf / PF_E].co[xf % PF_E], ent);
+      if (xb >= 0) store_chunks<sizeof(ent)>(((SweepRec<T>*)d.brec)[xb / PF_E].co[xb % PF_E], ent);
     }
     // the ghost state of a wall or symmetry face in the form the backward sweep's flux
     // increment takes it (its only ghost entries), so the sweep itself does no FP64 work
@@ -274,80 +290,147 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_sweep_prep(Dev d) {
   }
 }
 
-// ---- one cell of the forward sweep (wide schedule, stencil in cell-face order) ----
+// ---- one cell of the wide schedule (stencil in cell-face order) ----
+// A level is one launch of a few thousand cells at most, so its time is the latency of the
+// loads one cell waits for: the entries are taken WIDE_E at a time, their neighbours and
+// coefficients first, then all their increments together (an entry that does not apply reads
+// the cell's own). On 1470 polygons (10 levels, double-float) the forward sweep takes 66 us,
+// and took 133 us with one entry after the other.
+constexpr int WIDE_E = 4;
+template <class T>
+struct WideBatch {
+  int j[WIDE_E];
+  T co[WIDE_E][4], f[WIDE_E][8], w[WIDE_E][5];
+};
+// entries [k0, k0 + WIDE_E) of cell i, those below end; use(j): the entry needs increments
+template <class T, class Use>
+__device__ __forceinline__ void wide_load(WideBatch<T>& b, const Dev& d, const T* dF, const T* dWv, int i, int k0,
+                                          int end, Use use) {
+  const int n = d.nc_pad, nnz = d.nnz;
+  const T* sc = (const T*)d.sw_st;
+#pragma unroll
+  for (int e = 0; e < WIDE_E; e++) {
+    const int k = min(k0 + e, end - 1);
+    b.j[e] = d.sw_j[k];
+#pragma unroll
+    for (int q = 0; q < 4; q++) b.co[e][q] = sc[q * nnz + k];
+  }
+#pragma unroll
+  for (int e = 0; e < WIDE_E; e++) {
+    const int j = use(b.j[e]) ? b.j[e] : i;
+#pragma unroll
+    for (int q = 0; q < 8; q++) b.f[e][q] = dF[q * n + j];
+#pragma unroll
+    for (int v = 0; v < 5; v++) b.w[e][v] = dWv[v * n + j];
+  }
+}
+
+// the cell's increments and flux increments to global memory
+template <class T>
+__device__ __forceinline__ void wide_finish(const Dev& d, int i, const T* dw, T* dWv) {
+  const int n = d.nc_pad;
+  const T* c = (const T*)d.sw_cell;
+  T* dF = (T*)d.dF;
+  T o[8];
+  delta_flux<T>((T)d.W[i], (T)d.W[n + i], (T)d.W[2 * n + i], c[2 * n + i], c[3 * n + i], c[4 * n + i],
+                dw[0], dw[1], dw[2], dw[3], o);
+#pragma unroll
+  for (int v = 0; v < 5; v++) dWv[v * n + i] = dw[v];
+#pragma unroll
+  for (int q = 0; q < 8; q++) dF[q * n + i] = o[q];
+}
+
 template <class T>
 __device__ __forceinline__ void fwd_cell(const Dev& d, int i, bool sa_on) {
-  const int n = d.nc_pad, nnz = d.nnz;
+  const int n = d.nc_pad;
   T* dWs = (T*)d.dWs;
-  T* dF = (T*)d.dF;
+  const T* dF = (const T*)d.dF;
   const T* c = (const T*)d.sw_cell;
-  const T* sc = (const T*)d.sw_st;
   T acc[5];
 #pragma unroll
   for (int v = 0; v < 5; v++) acc[v] = (T)d.M[v * n + i];
-  for (int k = d.cf_ptr[i]; k < d.cf_ptr[i + 1]; k++) {
-    const int j = d.sw_j[k];
-    if (j < 0 || j >= i) continue;                   // ghost increments are zero forward
-    T f[8], w[5];
+  const int end = d.cf_ptr[i + 1];
+  for (int k0 = d.cf_ptr[i]; k0 < end; k0 += WIDE_E) {
+    auto use = [&](int j) { return j >= 0 && j < i; };   // ghost increments are zero forward
+    WideBatch<T> b;
+    wide_load<T>(b, d, dF, dWs, i, k0, end, use);
 #pragma unroll
-    for (int q = 0; q < 8; q++) f[q] = dF[q * n + j];
-#pragma unroll
-    for (int v = 0; v < 5; v++) w[v] = dWs[v * n + j];
-    fwd_acc<T>(acc, sc[k], sc[nnz + k], sc[2 * nnz + k], sc[3 * nnz + k], f, w, sa_on);
+    for (int e = 0; e < WIDE_E; e++)
+      if (k0 + e < end && use(b.j[e]))
+        fwd_acc<T>(acc, b.co[e][0], b.co[e][1], b.co[e][2], b.co[e][3], b.f[e], b.w[e], sa_on);
   }
   T dw[5];
 #pragma unroll
   for (int v = 0; v < 4; v++) dw[v] = inc_fwd<T>(acc[v], c[i]);
   dw[4] = sa_on ? inc_fwd<T>(acc[4], c[n + i]) : (T)0;
-#pragma unroll
-  for (int v = 0; v < 5; v++) dWs[v * n + i] = dw[v];
-  T o[8];
-  delta_flux<T>((T)d.W[i], (T)d.W[n + i], (T)d.W[2 * n + i], c[2 * n + i], c[3 * n + i], c[4 * n + i],
-                dw[0], dw[1], dw[2], dw[3], o);
-#pragma unroll
-  for (int q = 0; q < 8; q++) dF[q * n + i] = o[q];
+  wide_finish<T>(d, i, dw, dWs);
 }
 
 __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int bad);
 
-template <class T, int C>
-__device__ __forceinline__ void bwd_entry(const Dev& d, const T* ring, const T* dF, const T* dWo, int j, int slot,
-                                          const T* ws, T sx, T sy, T sl, T sa, bool sa_on, T* acc);
+template <class T>
+__device__ __forceinline__ T mn_x(T a, T fx, T b, T fy) { return fma_x(a, fx, mul_x(b, fy)); }
 
-// ---- one cell of the backward sweep (wide schedule, stencil in cell-face order) ----
+// The terms of a wall / symmetry ghost (face fc) in a cell's backward sum: the boundary map
+// of the cell's own forward increment ws and the flux increment about the ghost state give
+// t[0..3] (entry_sum of the four mean-flow components); returns the ghost's SA increment.
+template <class T>
+__device__ __forceinline__ T ghost_terms(const Dev& d, int fc, const T* ws, T sx, T sy, T sl, T* t) {
+  const int nf = d.nf;
+  T f[8], w[5];
+  w[0] = ws[0]; w[3] = ws[3];
+  if (d.fbc[fc] == 3 || d.fbc[fc] == 5) { w[1] = -ws[1]; w[2] = -ws[2]; w[4] = -ws[4]; }
+  else {
+    const T fx = (T)d.fnx[fc], fy = (T)d.fny[fc];
+    const T mn = mn_x(ws[1], fx, ws[2], fy);
+    const T mn2 = add_x(mn, mn);                                      // 2 (dm . n), exact
+    w[1] = fma_x(-mn2, fx, ws[1]); w[2] = fma_x(-mn2, fy, ws[2]); w[4] = ws[4];
+  }
+  const T* g = (const T*)d.gprim;   // ghost r, mx, my, u, v, H of this face (pre-pass)
+  delta_flux<T>(g[fc], g[nf + fc], g[2 * nf + fc], g[3 * nf + fc], g[4 * nf + fc], g[5 * nf + fc],
+                w[0], w[1], w[2], w[3], f);
+#pragma unroll
+  for (int v = 0; v < 4; v++) t[v] = entry_sum<T>(sx, sy, sl, f[2 * v], f[2 * v + 1], w[v]);
+  return w[4];
+}
+
 template <class T>
 __device__ __forceinline__ void bwd_cell(const Dev& d, int i, bool sa_on) {
-  const int n = d.nc_pad, nnz = d.nnz;
+  const int n = d.nc_pad;
   const T* dWs = (const T*)d.dWs;
   T* dWo = (T*)d.dW;
-  T* dF = (T*)d.dF;
+  const T* dF = (const T*)d.dF;
   const T* c = (const T*)d.sw_cell;
-  const T* sc = (const T*)d.sw_st;
   T ws[5];
 #pragma unroll
   for (int v = 0; v < 5; v++) ws[v] = dWs[v * n + i];
   T acc[5] = {0, 0, 0, 0, 0};
-  for (int k = d.cf_ptr[i]; k < d.cf_ptr[i + 1]; k++) {
-    int j = d.sw_j[k];
-    if (j >= 0) {
-      if (j <= i) continue;
-    } else {
-      const int f = d.cf_face[k];
-      if (d.fbc[f] == 1 || d.fbc[f] == 4) continue;  // free-stream and outflow increments are zero
-      j = -1 - f;
+  const int end = d.cf_ptr[i + 1];
+  for (int k0 = d.cf_ptr[i]; k0 < end; k0 += WIDE_E) {
+    auto use = [&](int j) { return j > i; };
+    WideBatch<T> b;
+    wide_load<T>(b, d, dF, dWo, i, k0, end, use);
+#pragma unroll
+    for (int e = 0; e < WIDE_E; e++) {
+      if (k0 + e >= end) continue;
+      if (use(b.j[e])) {
+        bwd_acc<T>(acc, b.co[e][0], b.co[e][1], b.co[e][2], b.co[e][3], b.f[e], b.w[e], sa_on);
+      } else if (b.j[e] < 0) {
+        const int f = d.cf_face[k0 + e];
+        if (d.fbc[f] == 1 || d.fbc[f] == 4) continue;  // free-stream and outflow increments are zero
+        T t[4];
+        const T w4 = ghost_terms<T>(d, f, ws, b.co[e][0], b.co[e][1], b.co[e][2], t);
+#pragma unroll
+        for (int v = 0; v < 4; v++) ghost_add<T>(acc[v], t[v]);
+        if (sa_on) bwd_sa<T>(acc[4], b.co[e][3], w4);
+      }
     }
-    bwd_entry<T, 1>(d, nullptr, dF, dWo, j, -1, ws, sc[k], sc[nnz + k], sc[2 * nnz + k], sc[3 * nnz + k], sa_on, acc);
   }
   T dw[5];
 #pragma unroll
-  for (int v = 0; v < 4; v++) { dw[v] = inc_bwd<T>(ws[v], acc[v], c[i]); dWo[v * n + i] = dw[v]; }
+  for (int v = 0; v < 4; v++) dw[v] = inc_bwd<T>(ws[v], acc[v], c[i]);
   dw[4] = sa_on ? inc_bwd<T>(ws[4], acc[4], c[n + i]) : (T)0;
-  dWo[4 * n + i] = dw[4];
-  T o[8];
-  delta_flux<T>((T)d.W[i], (T)d.W[n + i], (T)d.W[2 * n + i], c[2 * n + i], c[3 * n + i], c[4 * n + i],
-                dw[0], dw[1], dw[2], dw[3], o);
-#pragma unroll
-  for (int q = 0; q < 8; q++) dF[q * n + i] = o[q];
+  wide_finish<T>(d, i, dw, dWo);
 }
 
 // ---- state update W += dW (FP64), nu_tilde floor, Eq. 40 ratio, divergence check ----
@@ -414,29 +497,36 @@ __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int
   }
 }
 
-// ---- narrow schedule: one block per solve, shared-memory ring of recent increments ----
-// ring layout: [13][RING] of T: the 8 flux increments, then the 5 variable increments of
-// the cell at sweep position p (local to the solve), stored at slot p % RING.
+// ---- narrow schedule: one block (or a cluster) per solve, shared-memory ring ----
 //
-// Records. Each position has a static record (cell, neighbours, ring slots; 48 bytes) and
-// a per-iteration record (FwdDyn / BwdDyn: 128 bytes in FP32, 240 / 256 in FP64 and
-// double-float), both arrays of structures, so the records of one level are two contiguous
-// ranges. With one block per solve the block brings a level's records into shared memory
-// with two bulk copies (cp.async.bulk, the TMA engine's linear copy) completing on an
-// mbarrier, NST levels ahead; the cells' threads only wait on the barrier and read. With a
-// cluster of blocks per solve each thread stages its own record with 16-byte cp.async one
-// level ahead.
-template <class T>
-__device__ __forceinline__ void ring_put(T* ring, int slot, const T* o, const T* dw) {
-#pragma unroll
-  for (int q = 0; q < 8; q++) ring[q * RING + slot] = o[q];
-#pragma unroll
-  for (int v = 0; v < 5; v++) ring[(8 + v) * RING + slot] = dw[v];
-}
+// What bounds it: the latency of one cell's chain (neighbours' increments -> own increments
+// -> own flux increments) times the number of levels. A level holds 20-200 cells and a warp
+// with nobody beside it issues a dependent instruction every five cycles or so, so what
+// counts is the number of instructions of the busiest warp between two level barriers:
+//  - two threads per cell (lanes 2q, 2q + 1): lane 0 accumulates mass and x momentum and
+//    forms the x flux increments, lane 1 y momentum, energy and the y flux increments (both
+//    the SA row); they exchange the increments and one product by shuffles. Half the
+//    instructions per thread and twice the schedulers in use (FP64 issues one warp
+//    instruction per 64 cycles on a scheduler whatever its active lanes).
+//  - the cell warps do nothing else: a warp of its own issues the bulk copies that bring the
+//    records into shared memory (cp.async.bulk, chunks of 32 or 64 positions on an mbarrier each),
+//    other warps take the finished increments from the ring to global memory one level
+//    later and fetch the increments that left the ring ahead of their level. A cell's record
+//    is in registers when its level begins.
+//  - flux increments go to global memory only for the cells that a later cell reads there.
+//  - the ring holds the 13 values of a cell as 12 + 1: x fluxes, y fluxes and increments of
+//    the four mean-flow components (a lane reads its two of each with one vector load; 12
+//    values are 48 or 96 bytes, which puts consecutive cells on distinct banks), SA apart.
+// Forward + backward on the 20,480-cell hybrid plate (351 levels each way), against one
+// thread per cell that read its record inside the level and stored its results itself:
+// FP32 401 + 418 -> 195 + 209 us, double-float 592 + 719 -> 360 + 385, FP64 1192 + 1417 ->
+// 754 + 742 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
+// 60,160-cell O-mesh (605 levels; every level has a seam cell whose neighbour left the ring
+// 300 levels ago) FP32 946 + 895 -> 504 + 580 us.
 
 // With a cluster of C blocks per solve (C > 1), position q of the solve belongs to block
 // q % C and its increments sit in that block's ring, read through distributed shared
-// memory; RING is a multiple of C, so the slot q % RING names the owner too.
+// memory; the ring is a multiple of C, so the slot q % ring names the owner too.
 template <class T, int C>
 __device__ __forceinline__ const T* ring_of(const T* ring, int slot) {
   if constexpr (C == 1) {
@@ -448,80 +538,13 @@ __device__ __forceinline__ const T* ring_of(const T* ring, int slot) {
   }
 }
 
-template <class T, int C = 1>
-__device__ __forceinline__ void neighbour(const Dev& d, const T* ring, const T* dF, const T* dWv, int j, int slot,
-                                          T* f, T* w) {
-  const int n = d.nc_pad;
-  if (slot >= 0) {
-    const T* rb = ring_of<T, C>(ring, slot);
-#pragma unroll
-    for (int k = 0; k < 8; k++) f[k] = rb[k * RING + slot];
-#pragma unroll
-    for (int v = 0; v < 5; v++) w[v] = rb[(8 + v) * RING + slot];
-  } else {
-#pragma unroll
-    for (int k = 0; k < 8; k++) f[k] = dF[k * n + j];
-#pragma unroll
-    for (int v = 0; v < 5; v++) w[v] = dWv[v * n + j];
-  }
-}
+static_assert(sizeof(SweepRec<df64>) == sizeof(SweepRec<double>), "double-float records");
 
-// The increments of a record's PF_E entries. The ring reads of all entries are issued
-// together, unconditionally (an unused entry or one whose neighbour left the ring reads a
-// valid slot and its values are not used), so a cell waits for shared memory once rather
-// than once per entry; the rare neighbours that left the ring are then read from global
-// memory. Entries e >= cnt are not applied by the caller.
-template <class T, int C = 1>
-__device__ __forceinline__ void gather_entries(const Dev& d, const T* ring, const T* dF, const T* dWv, const int* j,
-                                               const int* slot, int cnt, T (*f)[8], T (*w)[5]) {
-#pragma unroll
-  for (int e = 0; e < PF_E; e++) {
-    const int sl = slot[e] >= 0 ? slot[e] : 0;
-    const T* rb = ring_of<T, C>(ring, sl);
-#pragma unroll
-    for (int k = 0; k < 8; k++) f[e][k] = rb[k * RING + sl];
-#pragma unroll
-    for (int v = 0; v < 5; v++) w[e][v] = rb[(8 + v) * RING + sl];
-  }
-  const int n = d.nc_pad;
-#pragma unroll
-  for (int e = 0; e < PF_E; e++)
-    if (e < cnt && slot[e] < 0 && j[e] >= 0) {
-#pragma unroll
-      for (int k = 0; k < 8; k++) f[e][k] = dF[k * n + j[e]];
-#pragma unroll
-      for (int v = 0; v < 5; v++) w[e][v] = dWv[v * n + j[e]];
-    }
-}
+// two or four consecutive values by vector loads / stores
+template <class T>
+struct alignas(2 * sizeof(T)) Pair { T a, b; };
 
-static_assert(sizeof(FwdDyn<df64>) == sizeof(FwdDyn<double>) && sizeof(BwdDyn<df64>) == sizeof(BwdDyn<double>),
-              "double-float records");
-
-// ---- asynchronous copies ----
-// 16-byte cp.async (cluster schedule): global -> shared in the background, no registers held
-__device__ __forceinline__ void cpa16(void* dst_smem, const void* src) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(dst_smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cpa_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// a record into registers with 16-byte loads (shared or global memory)
-template <class R>
-__device__ __forceinline__ R load_rec(const R* src) {
-  R r;
-#pragma unroll
-  for (int k = 0; k < (int)(sizeof(R) / 16); k++) reinterpret_cast<uint4*>(&r)[k] = reinterpret_cast<const uint4*>(src)[k];
-  return r;
-}
-
-template <class R>
-__device__ __forceinline__ void cpa_record(R* dst, const R* src) {   // sizeof(R) is a multiple of 16
-#pragma unroll
-  for (int k = 0; k < (int)(sizeof(R) / 16); k++) cpa16((char*)dst + 16 * k, (const char*)src + 16 * k);
-}
-
-// mbarrier and bulk copy (one block per solve)
+// mbarrier and bulk copy
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
 }
@@ -549,335 +572,527 @@ __device__ __forceinline__ void bulk_g2s(unsigned dst, const void* src, unsigned
                : "memory");
 }
 
-// ---- the work on one position (forward / backward), records in shared or global memory ----
-template <class T, int C = 1>
-__device__ __forceinline__ void fwd_process(const Dev& d, T* ring, int p, int pbase, const FwdStat& st,
-                                            const FwdDyn<T>& dy, bool sa_on) {
-  const int n = d.nc_pad;
-  T* dWs = (T*)d.dWs;
-  T* dF = (T*)d.dF;
-  T acc[5];
-#pragma unroll
-  for (int v = 0; v < 5; v++) acc[v] = dy.m[v];
-  const int cnt = st.cnt;
-  if (cnt >= 0) {
-    T f[PF_E][8], w[PF_E][5];
-    gather_entries<T, C>(d, ring, dF, dWs, st.j, st.slot, cnt, f, w);
-#pragma unroll
-    for (int e = 0; e < PF_E; e++)
-      if (e < cnt) fwd_acc<T>(acc, dy.co[e][0], dy.co[e][1], dy.co[e][2], dy.co[e][3], f[e], w[e], sa_on);
-  } else {
-    // more entries than the record holds: the position-ordered CSR stencil
-    const T* sc = (const T*)d.sc_f;
-    const int nfs = d.nfs;
-    for (int k = d.fs_ptr[p]; k < d.fs_ptr[p + 1]; k++) {
-      T f[8], w[5];
-      neighbour<T, C>(d, ring, dF, dWs, d.fs_j[k], d.fs_slot[k], f, w);
-      fwd_acc<T>(acc, sc[k], sc[nfs + k], sc[2 * nfs + k], sc[3 * nfs + k], f, w, sa_on);
-    }
-  }
-  T dw[5];
-#pragma unroll
-  for (int v = 0; v < 4; v++) dw[v] = inc_fwd<T>(acc[v], dy.c[0]);
-  dw[4] = sa_on ? inc_fwd<T>(acc[4], dy.c[1]) : (T)0;
-  T o[8];
-  delta_flux<T>(dy.w[0], dy.w[1], dy.w[2], dy.c[2], dy.c[3], dy.c[4], dw[0], dw[1], dw[2], dw[3], o);
-  const int slot = (p - pbase) % RING;
-  ring_put<T>(ring, slot, o, dw);
-  const int i = st.i;
-  BwdDyn<T>* rb = (BwdDyn<T>*)d.bdyn + st.pb;
-#pragma unroll
-  for (int v = 0; v < 5; v++) {
-    dWs[v * n + i] = dw[v];
-    rb->ws[v] = dw[v];                        // the backward sweep's copy of dW*
-  }
-#pragma unroll
-  for (int k = 0; k < 8; k++) dF[k * n + i] = o[k];
-}
-
+// shared memory: ring, side slots and the zero slot [12] | their SA increments | NREC records
+// | LVL_SMEM level offsets | an mbarrier per chunk | progress: levels finished | landed:
+// records in shared memory. A solve with a level wider than NREC - CHUNK positions, or a
+// cluster, reads its records and what left the ring from global memory. CHUNK: an FP32
+// level takes 0.5 us, so the copies come in fewer, larger pieces.
+constexpr int LVL_SMEM = 2048;
+constexpr int STORE_WARPS = 3;
 template <class T>
-__device__ __forceinline__ T mn_x(T a, T fx, T b, T fy) { return fma_x(a, fx, mul_x(b, fy)); }
-
-// the increments of a wall / symmetry ghost (face fc) in the backward sweep: the boundary
-// map of the cell's own forward increment ws, and the flux increment about the ghost state
-template <class T>
-__device__ __forceinline__ void ghost_entry(const Dev& d, int fc, const T* ws, T* f, T* w) {
-  const int nf = d.nf;
-  w[0] = ws[0]; w[3] = ws[3];
-  if (d.fbc[fc] == 3 || d.fbc[fc] == 5) { w[1] = -ws[1]; w[2] = -ws[2]; w[4] = -ws[4]; }
-  else {
-    const T fx = (T)d.fnx[fc], fy = (T)d.fny[fc];
-    const T mn = mn_x(ws[1], fx, ws[2], fy);
-    const T mn2 = add_x(mn, mn);                                      // 2 (dm . n), exact
-    w[1] = fma_x(-mn2, fx, ws[1]); w[2] = fma_x(-mn2, fy, ws[2]); w[4] = ws[4];
-  }
-  const T* g = (const T*)d.gprim;   // ghost r, mx, my, u, v, H of this face (pre-pass)
-  delta_flux<T>(g[fc], g[nf + fc], g[2 * nf + fc], g[3 * nf + fc], g[4 * nf + fc], g[5 * nf + fc],
-                w[0], w[1], w[2], w[3], f);
-}
-
-// contribution of one backward entry: upper neighbour j (its increments from the ring or
-// global memory), or a wall/symmetry ghost (j = -1 - face)
-template <class T, int C>
-__device__ __forceinline__ void bwd_entry(const Dev& d, const T* ring, const T* dF, const T* dWo, int j, int slot,
-                                          const T* ws, T sx, T sy, T sl, T sa, bool sa_on, T* acc) {
-  T f[8], w[5];
-  if (j >= 0) neighbour<T, C>(d, ring, dF, dWo, j, slot, f, w);
-  else ghost_entry<T>(d, -1 - j, ws, f, w);
-  bwd_acc<T>(acc, sx, sy, sl, sa, f, w, sa_on);
-}
-
-template <class T, int C = 1>
-__device__ __forceinline__ void bwd_process(const Dev& d, T* ring, int p, int pbase, const BwdStat& st,
-                                            const BwdDyn<T>& dy, bool sa_on) {
-  const int n = d.nc_pad;
-  T* dWo = (T*)d.dW;
-  T* dF = (T*)d.dF;
-  T ws[5];
-#pragma unroll
-  for (int v = 0; v < 5; v++) ws[v] = dy.ws[v];
-  T acc[5] = {0, 0, 0, 0, 0};
-  const int cnt = st.cnt;
-  if (cnt >= 0) {
-    T f[PF_E][8], w[PF_E][5];
-    gather_entries<T, C>(d, ring, dF, dWo, st.j, st.slot, cnt, f, w);
-#pragma unroll
-    for (int e = 0; e < PF_E; e++)
-      if (e < cnt && st.j[e] < 0) ghost_entry<T>(d, -1 - st.j[e], ws, f[e], w[e]);   // wall / symmetry ghost
-#pragma unroll
-    for (int e = 0; e < PF_E; e++)
-      if (e < cnt) bwd_acc<T>(acc, dy.co[e][0], dy.co[e][1], dy.co[e][2], dy.co[e][3], f[e], w[e], sa_on);
-  } else {
-    const T* sc = (const T*)d.sc_b;
-    const int nbs = d.nbs;
-    for (int k = d.bs_ptr[p]; k < d.bs_ptr[p + 1]; k++)
-      bwd_entry<T, C>(d, ring, dF, dWo, d.bs_j[k], d.bs_slot[k], ws, sc[k], sc[nbs + k], sc[2 * nbs + k],
-                      sc[3 * nbs + k], sa_on, acc);
-  }
-  T dw[5];
-#pragma unroll
-  for (int v = 0; v < 4; v++) dw[v] = inc_bwd<T>(ws[v], acc[v], dy.c[0]);
-  dw[4] = sa_on ? inc_bwd<T>(ws[4], acc[4], dy.c[1]) : (T)0;
-  T o[8];
-  delta_flux<T>(dy.w[0], dy.w[1], dy.w[2], dy.c[2], dy.c[3], dy.c[4], dw[0], dw[1], dw[2], dw[3], o);
-  ring_put<T>(ring, (p - pbase) % RING, o, dw);
-  const int i = st.i;
-#pragma unroll
-  for (int v = 0; v < 5; v++) dWo[v * n + i] = dw[v];
-#pragma unroll
-  for (int k = 0; k < 8; k++) dF[k * n + i] = o[k];
-}
-
-// ---- one block per solve: levels staged by bulk copies NST levels ahead ----
-constexpr int NST = 3;   // stage buffers (levels in flight)
-template <class T>
-__host__ __device__ constexpr int stage_max() { return sizeof(T) == 4 ? 256 : 128; }   // records per stage
-
-template <class T, bool FWD>
-struct Rec {
-  using Stat = typename std::conditional<FWD, FwdStat, BwdStat>::type;
-  using Dyn = typename std::conditional<FWD, FwdDyn<T>, BwdDyn<T>>::type;
+struct Smem {
+  static constexpr int SLOTS = ring_slots((int)sizeof(T)), ZERO = zero_slot((int)sizeof(T)), ALL = ZERO + 1;
+  static constexpr int CHUNK = sizeof(T) == 4 ? 64 : 32;
+  static constexpr int NREC = sizeof(T) == 4 ? 640 : 384;
+  static constexpr int NCHUNK = NREC / CHUNK;
+  static constexpr size_t ring4 = (size_t)12 * ALL * sizeof(T);
+  static constexpr size_t rec = (ring4 + (size_t)ALL * sizeof(T) + 15) / 16 * 16;
+  static constexpr size_t lvl = rec + (size_t)NREC * sizeof(SweepRec<T>);
+  static constexpr size_t bar = lvl + (size_t)LVL_SMEM * sizeof(int);
+  static constexpr size_t flag = bar + 8 * (size_t)NCHUNK;
+  static constexpr size_t total = flag + 16;
+  static_assert(2 * (NREC - CHUNK) <= SLOTS, "two staged levels fit the ring");
+  static_assert(total <= 232448, "shared memory of one block");
 };
 
-// dynamic shared memory: ring | NST x stage_max static records | NST x stage_max dynamic
-// records | NST mbarriers | abort flag
-template <class T, bool FWD>
-__host__ __device__ constexpr size_t stage_stat_off() { return (size_t)13 * RING * sizeof(T); }
-template <class T, bool FWD>
-__host__ __device__ constexpr size_t stage_dyn_off() {
-  return stage_stat_off<T, FWD>() + (size_t)NST * stage_max<T>() * sizeof(typename Rec<T, FWD>::Stat);
-}
-template <class T, bool FWD>
-__host__ __device__ constexpr size_t stage_bar_off() {
-  return stage_dyn_off<T, FWD>() + (size_t)NST * stage_max<T>() * sizeof(typename Rec<T, FWD>::Dyn);
-}
-template <class T, bool FWD>
-__host__ __device__ constexpr size_t bulk_smem() { return stage_bar_off<T, FWD>() + 8 * NST + 16; }
+// what a thread holds of its cell's record: the sum's start (a0, a1, a4: forward the
+// residual), backward the forward increments (m0, m1, m4), constants, two entries
+template <class T>
+struct LaneRec {
+  int i, kind, pb, spill;
+  int slot[PF_E];
+  T a0, a1, a4, m0, m1, m4, r, mx, my, c0, c1, u, v, H;
+  T co[2][4];       // quads and triangles mostly have no more
+};
 
-// issue the bulk copies of level [b, e) (its first stage_max records) into stage k
-template <class T, bool FWD>
-__device__ __forceinline__ void stage_level(const Dev& d, unsigned char* smem, int k, int b, int e) {
-  using Stat = typename Rec<T, FWD>::Stat;
-  using Dyn = typename Rec<T, FWD>::Dyn;
-  const int nrec = min(e - b, stage_max<T>());
-  const unsigned bar = (unsigned)__cvta_generic_to_shared(smem + stage_bar_off<T, FWD>() + 8 * k);
-  const unsigned ss = (unsigned)__cvta_generic_to_shared(smem + stage_stat_off<T, FWD>()) +
-                      (unsigned)(k * stage_max<T>() * sizeof(Stat));
-  const unsigned sd = (unsigned)__cvta_generic_to_shared(smem + stage_dyn_off<T, FWD>()) +
-                      (unsigned)(k * stage_max<T>() * sizeof(Dyn));
-  const Stat* gs = (FWD ? (const Stat*)d.fst : (const Stat*)d.bst) + b;
-  const Dyn* gd = (const Dyn*)(FWD ? d.fdyn : d.bdyn) + b;
-  mbar_expect(bar, (unsigned)(nrec * (sizeof(Stat) + sizeof(Dyn))));
-  bulk_g2s(ss, gs, (unsigned)(nrec * sizeof(Stat)), bar);
-  bulk_g2s(sd, gd, (unsigned)(nrec * sizeof(Dyn)), bar);
+template <class T>
+__device__ __forceinline__ void load_co(T* o, const T* co) {
+#pragma unroll
+  for (int k = 0; k < (int)(4 * sizeof(T) / 16); k++)
+    reinterpret_cast<uint4*>(o)[k] = reinterpret_cast<const uint4*>(co)[k];
 }
 
-// The sweep of one solve by one block. Level l (k = l - l0) sits in stage k % NST, phase
-// (k / NST) & 1 of its barrier. Thread 0 issues the copies; every thread waits for its
-// level's barrier (at most wait_limit tries: a wait that runs out marks the solve
-// IGKS_TIMEOUT, the block stops after the level barrier, waits for its copies in flight,
-// and the update leaves the solve's state untouched). Positions beyond stage_max of a wide
-// level read their records from global memory.
 template <class T, bool FWD>
-__device__ __forceinline__ void sweep_bulk(const Dev& d) {
-  using Stat = typename Rec<T, FWD>::Stat;
-  using Dyn = typename Rec<T, FWD>::Dyn;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* ring = (T*)smem_raw;
-  const Stat* sst = (const Stat*)(smem_raw + stage_stat_off<T, FWD>());
-  const Dyn* sdy = (const Dyn*)(smem_raw + stage_dyn_off<T, FWD>());
-  const unsigned bar0 = (unsigned)__cvta_generic_to_shared(smem_raw + stage_bar_off<T, FWD>());
-  volatile int* abort_flag = (volatile int*)(smem_raw + stage_bar_off<T, FWD>() + 8 * NST);
-  const int s = d.g_solve0 + blockIdx.x;
-  if (d.st[s].state != 0 || d.flow[s].scheme == 1) return;
-  if (!FWD && d.tmo[s]) return;                       // the forward sweep of this solve gave up
-  const bool sa_on = d.flow[s].sa_on;
-  const int* lvl = FWD ? d.fwd_lvl : d.bwd_lvl;
-  const int* lsp = FWD ? d.lvl_solve_ptr : d.blvl_solve_ptr;
-  const int l0 = lsp[s], l1 = lsp[s + 1] - 1, nl = l1 - l0;
-  if (nl <= 0) return;
-  const Stat* gst = FWD ? (const Stat*)d.fst : (const Stat*)d.bst;
-  const Dyn* gdy = (const Dyn*)(FWD ? d.fdyn : d.bdyn);
-  const int limit = d.wait_limit;
-  const int tid = threadIdx.x;
-  int issued = 0;                                     // levels issued (thread 0)
-  int nb = 0;                                         // offset of the next level to issue (thread 0)
-  if (tid == 0) {
-    for (int k = 0; k < NST; k++) mbar_init(bar0 + 8 * k, 1);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    nb = lvl[l0];
-    for (; issued < NST && issued < nl; issued++) {
-      const int e = lvl[l0 + issued + 1];
-      if (!(FWD && d.starve_test && issued == 1)) stage_level<T, FWD>(d, smem_raw, issued, nb, e);
-      nb = e;
+__device__ __forceinline__ void load_rec(LaneRec<T>& o, const SweepRec<T>* dy, int lane) {
+  const int4 b = *reinterpret_cast<const int4*>(dy->st.slot), a = *reinterpret_cast<const int4*>(&dy->st);
+  o.slot[0] = b.x; o.slot[1] = b.y; o.slot[2] = b.z;
+  o.i = a.x; o.kind = a.y; o.pb = a.z; o.spill = a.w;
+  const Pair<T> m = *reinterpret_cast<const Pair<T>*>(&dy->m[2 * lane]);
+  constexpr int N = sizeof(T) == 4 ? 12 : 10;           // m[4], w[3], c[5], pad0[0]: whole chunks
+  alignas(16) T q[N];
+#pragma unroll
+  for (int k = 0; k < (int)(N * sizeof(T) / 16); k++)
+    reinterpret_cast<uint4*>(q)[k] = reinterpret_cast<const uint4*>(&dy->m[4])[k];
+  if constexpr (FWD) {
+    o.a0 = m.a; o.a1 = m.b; o.a4 = q[0];
+  } else {
+    const Pair<T> s = *reinterpret_cast<const Pair<T>*>(&dy->start[2 * lane]);
+    o.a0 = s.a; o.a1 = s.b; o.a4 = q[9];
+    o.m0 = m.a; o.m1 = m.b; o.m4 = q[0];
+  }
+  o.r = q[1]; o.mx = q[2]; o.my = q[3];
+  o.c0 = q[4]; o.c1 = q[5]; o.u = q[6]; o.v = q[7]; o.H = q[8];
+#pragma unroll
+  for (int e = 0; e < 2; e++) load_co<T>(o.co[e], dy->co[e]);
+}
+
+// one stencil entry as a lane needs it: x and y flux increments and increments of its two
+// components, and the SA increment
+template <class T>
+struct LaneNb { T x0, x1, y0, y1, w0, w1, w4; };
+
+template <class T, int C>
+__device__ __forceinline__ void ring_read(LaneNb<T>& o, const T* ring, const T* ring4, int slot, int lane) {
+  const T* b = ring_of<T, C>(ring, slot) + slot * 12 + 2 * lane;
+  const Pair<T> x = *reinterpret_cast<const Pair<T>*>(b), y = *reinterpret_cast<const Pair<T>*>(b + 4),
+                w = *reinterpret_cast<const Pair<T>*>(b + 8);
+  o.x0 = x.a; o.x1 = x.b; o.y0 = y.a; o.y1 = y.b; o.w0 = w.a; o.w1 = w.b;
+  o.w4 = ring_of<T, C>(ring4, slot)[slot];
+}
+
+template <class T>
+__device__ __forceinline__ void global_read(LaneNb<T>& o, const Dev& d, const T* dWv, int j, int lane) {
+  const int n = d.nc_pad;
+  const T* dF = (const T*)d.dF;
+  o.x0 = dF[(4 * lane) * n + j]; o.y0 = dF[(4 * lane + 1) * n + j];
+  o.x1 = dF[(4 * lane + 2) * n + j]; o.y1 = dF[(4 * lane + 3) * n + j];
+  o.w0 = dWv[(2 * lane) * n + j]; o.w1 = dWv[(2 * lane + 1) * n + j]; o.w4 = dWv[4 * n + j];
+}
+
+// a lane's results for one cell: its increments (w4: the SA row, both lanes) and the four
+// mean-flow components of its flux direction
+template <class T>
+struct LaneOut { T w0, w1, w4, f[4]; };
+
+template <class T>
+__device__ __forceinline__ T shfl_pair(T x) { return __shfl_xor_sync(0xffffffffu, x, 1); }
+template <>
+__device__ __forceinline__ df64 shfl_pair<df64>(df64 x) {
+  return df64(__shfl_xor_sync(0xffffffffu, x.hi, 1), __shfl_xor_sync(0xffffffffu, x.lo, 1));
+}
+
+// The increments and flux increments of one cell from its accumulators; the same operations
+// as delta_flux, split over the two lanes. Called by whole warps.
+template <class T, bool FWD>
+__device__ __forceinline__ LaneOut<T> lane_finish(const LaneRec<T>& rc, T acc0, T acc1, T acc4, int lane, bool sa_on) {
+  LaneOut<T> o;
+  if constexpr (FWD) {
+    o.w0 = inc_fwd<T>(acc0, rc.c0); o.w1 = inc_fwd<T>(acc1, rc.c0);
+    o.w4 = sa_on ? inc_fwd<T>(acc4, rc.c1) : (T)0;
+  } else {
+    o.w0 = inc_bwd<T>(rc.m0, acc0, rc.c0); o.w1 = inc_bwd<T>(rc.m1, acc1, rc.c0);
+    o.w4 = sa_on ? inc_bwd<T>(rc.m4, acc4, rc.c1) : (T)0;
+  }
+  const T p0 = shfl_pair(o.w0), p1 = shfl_pair(o.w1);
+  const T dr = lane ? p0 : o.w0, dE = lane ? o.w1 : p1;
+  const T dm = lane ? o.w0 : o.w1, dmo = lane ? p1 : p0;         // momentum along / across the lane's direction
+  const T vel = lane ? rc.v : rc.u, mom = lane ? rc.my : rc.mx, mo = lane ? rc.mx : rc.my;
+  const T inv1 = rcp_x(add_x(rc.r, dr));
+  const T dv = mul_x(fma_x(-vel, dr, dm), inv1);
+  const T v1 = add_x(vel, dv);
+  const T q = fma_x(dm, v1, mul_x(mom, dv));
+  const T dp = mul_x((T)(GAMMA - 1.0), fma_x((T)(-0.5), add_x(q, shfl_pair(q)), dE));
+  const T dH = add_x(dE, dp);
+  const T own = add_x(q, dp), cross = fma_x(dmo, v1, mul_x(mo, dv));
+  o.f[0] = dm;
+  o.f[1] = lane ? cross : own;
+  o.f[2] = lane ? own : cross;
+  o.f[3] = fma_x(dH, v1, mul_x(rc.H, dv));
+  return o;
+}
+
+template <class T>
+__device__ __forceinline__ void ring_put(T* ring, T* ring4, int slot, const LaneOut<T>& o, int lane) {
+  T* b = ring + slot * 12;
+  Pair<T>* f = reinterpret_cast<Pair<T>*>(b + 4 * lane);
+  f[0] = Pair<T>{o.f[0], o.f[1]};
+  f[1] = Pair<T>{o.f[2], o.f[3]};
+  *reinterpret_cast<Pair<T>*>(b + 8 + 2 * lane) = Pair<T>{o.w0, o.w1};
+  if (lane) ring4[slot] = o.w4;
+}
+
+// increments to global memory: the forward one into the cell's backward record (at = its
+// position), the backward one into dW (at = the cell)
+template <class T, bool FWD>
+__device__ __forceinline__ void store_inc(const Dev& d, int at, const T* w, T w4) {
+  if constexpr (FWD) {
+    T* m = ((SweepRec<T>*)d.brec + at)->m;
+    reinterpret_cast<Pair<T>*>(m)[0] = Pair<T>{w[0], w[1]};
+    reinterpret_cast<Pair<T>*>(m)[1] = Pair<T>{w[2], w[3]};
+    m[4] = w4;
+  } else {
+    const int n = d.nc_pad;
+    T* dWo = (T*)d.dW;
+#pragma unroll
+    for (int v = 0; v < 4; v++) dWo[v * n + at] = w[v];
+    dWo[4 * n + at] = w4;
+  }
+}
+
+// the increments of a cell that a later one reads from global memory (before the barrier)
+template <class T, bool FWD>
+__device__ __noinline__ void store_spill(const Dev& d, int i, LaneOut<T> o, int lane) {
+  const int n = d.nc_pad;
+  T* dWv = (T*)(FWD ? d.dWs : d.dW);
+  T* dF = (T*)d.dF;
+  dWv[(2 * lane) * n + i] = o.w0;
+  dWv[(2 * lane + 1) * n + i] = o.w1;
+  if (lane) dWv[4 * n + i] = o.w4;
+  for (int v = 0; v < 4; v++) dF[(2 * v + lane) * n + i] = o.f[v];
+}
+
+// the accumulators of a cell with more entries than a record holds (p: its position)
+template <class T, bool FWD, int C>
+__device__ __noinline__ void csr_sum(const Dev& d, const T* ring, const T* ring4, int slots, int p, int lane, bool sa_on, T* acc) {
+  const T* sc = (const T*)(FWD ? d.sc_f : d.sc_b);
+  const int ne = FWD ? d.nfs : d.nbs;
+  const int* ptr = FWD ? d.fs_ptr : d.bs_ptr;
+  const int* sj = FWD ? d.fs_j : d.bs_j;
+  const int* ss = FWD ? d.fs_slot : d.bs_slot;
+  for (int k = ptr[p]; k < ptr[p + 1]; k++) {
+    const T sx = sc[k], sy = sc[ne + k], sl = sc[2 * ne + k], sa = sc[3 * ne + k];
+    if (!FWD && ss[k] == SLOT_GHOST) {
+      const T* ws = ((const SweepRec<T>*)d.brec)[p].m;
+      T t[4];
+      const T w4 = ghost_terms<T>(d, -1 - sj[k], ws, sx, sy, sl, t);
+      ghost_add<T>(acc[0], lane ? t[2] : t[0]);
+      ghost_add<T>(acc[1], lane ? t[3] : t[1]);
+      if (sa_on) bwd_sa<T>(acc[2], sa, w4);
+      continue;
+    }
+    LaneNb<T> b;
+    if ((unsigned)ss[k] < (unsigned)slots) ring_read<T, C>(b, ring, ring4, ss[k], lane);
+    else global_read<T>(b, d, (const T*)(FWD ? d.dWs : d.dW), sj[k], lane);
+    if constexpr (FWD) {
+      fwd_comp<T>(acc[0], sx, sy, sl, b.x0, b.y0, b.w0);
+      fwd_comp<T>(acc[1], sx, sy, sl, b.x1, b.y1, b.w1);
+      if (sa_on) fwd_sa<T>(acc[2], sa, b.w4);
+    } else {
+      bwd_comp<T>(acc[0], sx, sy, sl, b.x0, b.y0, b.w0);
+      bwd_comp<T>(acc[1], sx, sy, sl, b.x1, b.y1, b.w1);
+      if (sa_on) bwd_sa<T>(acc[2], sa, b.w4);
     }
   }
-  __syncthreads();
-  const int pbase = lvl[l0];
-  int b = lvl[l0], e = lvl[l0 + 1];
-  int k = 0;
-  for (; k < nl; k++) {
-    const int l = l0 + k;
-    const int en = (k + 1 < nl) ? lvl[l + 2] : e;     // next level's end, loaded a level early
-    const int st_k = k % NST;
-    const int nnext = (tid == 0 && issued < nl) ? lvl[l0 + issued + 1] : 0;   // for the copy issued below
-    const bool mine = b + tid < e;
-    bool ok = true;
-    if (mine) ok = mbar_wait(bar0 + 8 * st_k, (unsigned)((k / NST) & 1), limit);
-    if (!ok) {
-      d.tmo[s] = 1;
-      *abort_flag = 1;
-    } else {
-      const int smax = stage_max<T>();
-      for (int p = b + tid; p < e; p += blockDim.x) {
-        const int q = p - b;
-        Stat cs;
-        Dyn cd;
-        if (q < smax) {              // staged: shared-memory loads
-          cs = load_rec(sst + st_k * smax + q);
-          cd = load_rec(sdy + st_k * smax + q);
-        } else {
-          cs = load_rec(gst + p);
-          cd = load_rec(gdy + p);
-        }
-        if constexpr (FWD) fwd_process<T>(d, ring, p, pbase, cs, cd, sa_on);
-        else bwd_process<T>(d, ring, p, pbase, cs, cd, sa_on);
+}
+
+// one interior entry applied to the accumulators
+template <class T, bool FWD>
+__device__ __forceinline__ void apply_entry(T& a0, T& a1, T& a4, const T* co, const LaneNb<T>& b, bool sa_on) {
+  if constexpr (FWD) {
+    fwd_comp<T>(a0, co[0], co[1], co[2], b.x0, b.y0, b.w0);
+    fwd_comp<T>(a1, co[0], co[1], co[2], b.x1, b.y1, b.w1);
+    if (sa_on) fwd_sa<T>(a4, co[3], b.w4);
+  } else {
+    bwd_comp<T>(a0, co[0], co[1], co[2], b.x0, b.y0, b.w0);
+    bwd_comp<T>(a1, co[0], co[1], co[2], b.x1, b.y1, b.w1);
+    if (sa_on) bwd_sa<T>(a4, co[3], b.w4);
+  }
+}
+
+// a ghost entry behind an interior one (backward): ready terms in the entry's coefficients,
+// the signed SA coefficient in the face's first ghost value
+template <class T>
+__device__ __forceinline__ void apply_ghost(const Dev& d, T& a0, T& a1, T& a4, const T* co, int j, T m4, int lane,
+                                            bool sa_on) {
+  ghost_add<T>(a0, lane ? co[2] : co[0]);
+  ghost_add<T>(a1, lane ? co[3] : co[1]);
+  if (sa_on) bwd_sa<T>(a4, ((const T*)d.gprim)[-1 - j], m4);
+}
+
+// The increments of the cell at position p (its record in rc; co: the record's coefficients
+// in memory). rare: the kinds that take the general path (with the side slots' when the solve
+// is not staged). Called by whole warps; a thread without a cell of its own (valid = false) works
+// on a copy of another's and stores nothing.
+template <class T, bool FWD, int C>
+__device__ __forceinline__ LaneOut<T> lane_cell(const Dev& d, T* ring, T* ring4, int rare, const LaneRec<T>& rc,
+                                                const T* co, int p, int slot, int lane, bool valid, bool sa_on) {
+  T acc0 = rc.a0, acc1 = rc.a1, acc4 = rc.a4;
+  LaneNb<T> nb[2];
+#pragma unroll
+  for (int e = 0; e < 2; e++) ring_read<T, C>(nb[e], ring, ring4, max(rc.slot[e], 0), lane);
+  if (!(rc.kind & rare)) {
+#pragma unroll
+    for (int e = 0; e < 2; e++) apply_entry<T, FWD>(acc0, acc1, acc4, rc.co[e], nb[e], sa_on);
+  } else if (!(rc.kind & KIND_CSR)) {
+    const int* js = (FWD ? d.fj : d.bj)[p].j;
+    const int slots = rare & KIND_SIDE ? Smem<T>::SLOTS : Smem<T>::ALL;
+#pragma unroll 1
+    for (int e = 0; e < (rc.kind & KIND_COUNT); e++) {
+      const int sl = e == 0 ? rc.slot[0] : e == 1 ? rc.slot[1] : rc.slot[2];
+      alignas(16) T c[4];
+      load_co<T>(c, co + 4 * e);
+      if (!FWD && sl == SLOT_GHOST) {
+        apply_ghost<T>(d, acc0, acc1, acc4, c, js[e], rc.m4, lane, sa_on);
+        continue;
+      }
+      LaneNb<T> b;
+      if ((unsigned)sl < (unsigned)slots) ring_read<T, C>(b, ring, ring4, sl, lane);
+      else global_read<T>(b, d, (const T*)(FWD ? d.dWs : d.dW), js[e], lane);
+      apply_entry<T, FWD>(acc0, acc1, acc4, c, b, sa_on);
+    }
+  } else {
+    T acc[3] = {FWD ? acc0 : (T)0, FWD ? acc1 : (T)0, FWD ? acc4 : (T)0};
+    csr_sum<T, FWD, C>(d, ring, ring4, rare & KIND_SIDE ? Smem<T>::SLOTS : Smem<T>::ALL, p, lane, sa_on, acc);
+    acc0 = acc[0]; acc1 = acc[1]; acc4 = acc[2];
+  }
+  __syncwarp();
+  const LaneOut<T> o = lane_finish<T, FWD>(rc, acc0, acc1, acc4, lane, sa_on);
+  if (valid) {
+    ring_put<T>(ring, ring4, slot, o, lane);
+    if (rc.spill) store_spill<T, FWD>(d, rc.i, o, lane);
+  }
+  return o;
+}
+
+// the first position at or after b that belongs to cluster block r (positions q are dealt
+// round the C blocks: q % C == r)
+template <int C>
+__device__ __forceinline__ int first_own(int b, int r) {
+  return b + ((r - b) & (C - 1));
+}
+
+// The forward sweep's last step: what the wall and symmetry ghosts add to the backward sums
+// (they need the cells' own forward increments only). Ghosts that come first in a cell's
+// order make the sum's start, in the same additions; later ones leave their terms in their
+// entries.
+template <class T>
+__device__ __forceinline__ void ghost_pass(const Dev& d, int s, int first, int step, bool sa_on) {
+  const T* sc = (const T*)d.sc_b;
+  const int g1 = d.gent_ptr[s + 1], nbs = d.nbs;
+  for (int g = d.gent_ptr[s] + first; g < g1; g += step) {
+    const int p = d.gent_pos[g];
+    SweepRec<T>* rec = (SweepRec<T>*)d.brec + p;
+    T ws[5], t[4], a[4] = {(T)0, (T)0, (T)0, (T)0}, a4 = (T)0;
+#pragma unroll
+    for (int v = 0; v < 5; v++) ws[v] = rec->m[v];
+    int lead = -1;                                     // entries before the first interior one
+    for (int k = d.bs_ptr[p]; k < d.bs_ptr[p + 1]; k++) {
+      if (d.bs_slot[k] != SLOT_GHOST) {
+        if (lead < 0) lead = k - d.bs_ptr[p];
+        continue;
+      }
+      const int f = -1 - d.bs_j[k];
+      const T sa = sc[3 * nbs + k];
+      const T w4 = ghost_terms<T>(d, f, ws, sc[k], sc[nbs + k], sc[2 * nbs + k], t);
+      if (lead < 0) {
+#pragma unroll
+        for (int v = 0; v < 4; v++) ghost_add<T>(a[v], t[v]);
+        if (sa_on) bwd_sa<T>(a4, sa, w4);
+      } else {
+        T* co = rec->co[k - d.bs_ptr[p] - lead];
+#pragma unroll
+        for (int v = 0; v < 4; v++) co[v] = t[v];
+        ((T*)d.gprim)[f] = d.fbc[f] == 2 ? sa : -sa;   // the face's ghost values have been used
       }
     }
-    __syncthreads();                                  // level done; stage st_k is free
-    if (*abort_flag) break;
-    if (tid == 0 && issued < nl) {
-      // the stage was read by generic loads: order those before the async proxy's writes
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      stage_level<T, FWD>(d, smem_raw, issued % NST, nb, nnext);
-      nb = nnext;
-      issued++;
-    }
-    b = e;
-    e = en;
+#pragma unroll
+    for (int v = 0; v < 4; v++) rec->start[v] = a[v];
+    rec->pad0[0] = a4;
   }
-  // after a wait ran out: let the copies already issued land before the block exits
-  if (tid == 0 && k < nl)
-    for (int kk = k; kk < issued; kk++)
-      if (!(FWD && d.starve_test && kk == 1)) mbar_wait(bar0 + 8 * (kk % NST), (unsigned)((kk / NST) & 1), limit);
 }
 
-template <class T>
-__global__ void __launch_bounds__(NARROW_THREADS) k_sweep_fwd_bulk(Dev d) { sweep_bulk<T, true>(d); }
-template <class T>
-__global__ void __launch_bounds__(NARROW_THREADS) k_sweep_bwd_bulk(Dev d) { sweep_bulk<T, false>(d); }
+// level barrier of the cell and store warps
+__device__ __forceinline__ void bar_levels(int threads) {
+  asm volatile("bar.sync 1, %0;\n" ::"r"(threads) : "memory");
+}
+__device__ __forceinline__ int ld_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.cta.shared.s32 %0, [%1];\n" : "=r"(v) : "r"((unsigned)__cvta_generic_to_shared(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(int* p, int v) {
+  asm volatile("st.release.cta.shared.s32 [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+}
 
-// ---- a cluster of C blocks per solve: positions dealt round the blocks, records staged
-// per thread with 16-byte cp.async one level ahead ----
-// the first position at or after b that belongs to cluster block r (positions q = p - pbase
-// are dealt round the C blocks: q % C == r)
-template <int C>
-__device__ __forceinline__ int first_own(int b, int pbase, int r) {
-  return b + (((r - (b - pbase)) % C) + C) % C;
+// The sweep of one solve. Positions q are counted from the solve's first; level k is
+// [lv(k), lv(k + 1)). With one block per solve the warps have roles:
+//  - cell warps: two threads per cell of level k; then they read the records of level k + 1
+//    (from shared memory as far as they have landed, the others from global memory);
+//  - store warps: the increments of level k to global memory during level k + 1 (their ring
+//    slots are not reused before level k + 2: two levels fit the ring); the first of them
+//    also fetches increments that left the ring: it reads them during level k for level
+//    k + 2 and puts them into the side slots during level k + 1;
+//  - the copy warp: a chunk's buffer is free once all its positions lie in finished levels;
+//    it issues chunks as buffers become free and counts the records that have landed. It
+//    runs beside the level barriers, and nobody waits for it. A chunk that has not landed
+//    after wait_limit tries marks the solve IGKS_TIMEOUT (the update leaves its state
+//    untouched); the warp then waits for the other copies in flight and ends.
+template <class T, bool FWD, int C>
+__device__ __forceinline__ void sweep_narrow(const Dev& d) {
+  using S = Smem<T>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* ring = (T*)smem_raw;
+  T* ring4 = (T*)(smem_raw + S::ring4);
+  const SweepRec<T>* srec = (const SweepRec<T>*)(smem_raw + S::rec);
+  int* slv = (int*)(smem_raw + S::lvl);
+  const unsigned bar0 = (unsigned)__cvta_generic_to_shared(smem_raw + S::bar);
+  int* progress = (int*)(smem_raw + S::flag);
+  int* landed_p = progress + 1;
+  const int s = d.g_solve0 + blockIdx.x / C, r = blockIdx.x % C;   // one cluster of C blocks per solve
+  if (d.st[s].state != 0 || d.flow[s].scheme == 1) return;         // uniform over the cluster
+  if (!FWD && d.tmo[s]) return;                                    // the forward sweep of this solve gave up
+  // (without SA its coefficients and 1/a_ii are zero and so are its increments: on the FP32
+  // pipes the row is computed all the same, which costs less than the branches)
+  const bool sa_on = std::is_same<T, double>::value ? d.flow[s].sa_on != 0 : true;
+  const int* glv = FWD ? d.fwd_lvl : d.bwd_lvl;
+  const int* lsp = FWD ? d.lvl_solve_ptr : d.blvl_solve_ptr;
+  const int l0 = lsp[s], nl = lsp[s + 1] - 1 - l0;
+  if (nl <= 0) return;
+  glv += l0;
+  const int pbase = glv[0], np = glv[nl] - pbase;
+  const SweepRec<T>* grec = (const SweepRec<T>*)(FWD ? d.frec : d.brec) + pbase;
+  const int tid = threadIdx.x;
+  const int nct = C == 1 ? (int)blockDim.x - 32 * (STORE_WARPS + 1) : (int)blockDim.x;   // cell threads
+  const bool lvs = nl + 3 < LVL_SMEM;                              // level offsets in shared memory
+  int wide = 0;
+  for (int k = tid; k <= nl + 2; k += blockDim.x) {
+    const int v = glv[min(k, nl)] - pbase;
+    if (lvs) slv[k] = v;
+    if (k > 0) wide |= (v - (glv[min(k - 1, nl)] - pbase)) > S::NREC - S::CHUNK;
+  }
+  if (C == 1 && tid < S::NCHUNK) mbar_init(bar0 + 8 * tid, 1);
+  if (C == 1) asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  if (tid == 0) { *progress = 0; *landed_p = 0; }
+  if (tid < 13) (tid < 12 ? ring + 12 * S::ZERO : ring4 + S::ZERO - 12)[tid] = (T)0;
+  const bool staged = !__syncthreads_or(wide) && C == 1;
+  if constexpr (C > 1) cg::this_cluster().sync();                  // every block runs before any remote read
+  auto lv = [&](int k) { return lvs ? slv[k] : glv[min(k, nl)] - pbase; };
+
+  if (tid < nct) {
+    const int lane = tid & 1, w0 = (tid & 31) / 2 * C, own = C * (tid >> 1), step = C * nct / 2;
+    const int rare = staged ? KIND_RARE : KIND_RARE | KIND_SIDE;
+    LaneRec<T> rc;
+    auto fetch = [&](int q, int landed) {
+      if (q < landed) load_rec<T, FWD>(rc, srec + q % S::NREC, lane);
+      else load_rec<T, FWD>(rc, grec + q, lane);
+    };
+    int e = lv(1), en = lv(2), q = first_own<C>(0, r) + own;
+    if (q - w0 < e) fetch(min(q, e - 1), 0);                       // a warp works if its first cell exists
+    for (int k = 0; k < nl; k++) {
+      const int ef = lv(k + 3);
+      const int landed = C == 1 ? ld_acquire(landed_p) : 0;
+      while (q - w0 < e) {               // more than one round in a level wider than the block
+        const bool valid = q < e;
+        const int qc = min(q, e - 1);
+        const T* co = qc < landed ? srec[qc % S::NREC].co[0] : grec[qc].co[0];
+        const LaneOut<T> o = lane_cell<T, FWD, C>(d, ring, ring4, rare, rc, co, pbase + qc, q & (S::SLOTS - 1), lane,
+                                                  valid, sa_on);
+        if (C > 1 || !staged) {          // no store warps, or levels that may overrun the ring
+          const T p0 = shfl_pair(o.w0), p1 = shfl_pair(o.w1);
+          const T w[4] = {o.w0, o.w1, p0, p1};
+          if (valid && lane == 0) store_inc<T, FWD>(d, FWD ? rc.pb : rc.i, w, o.w4);
+        }
+        q += step;
+        if (q - w0 < e) fetch(min(q, e - 1), landed);
+      }
+      q = first_own<C>(e, r) + own;
+      if (q - w0 < en) fetch(min(q, en - 1), landed);
+      if constexpr (C == 1) bar_levels(nct + 32 * STORE_WARPS);
+      else cg::this_cluster().sync();    // release/acquire over the cluster's shared and global writes
+      e = en; en = ef;
+    }
+  } else if (tid < nct + 32 * STORE_WARPS) {
+    const int t = tid - nct, n = d.nc_pad;
+    const int* sp = (FWD ? d.fside_ptr : d.bside_ptr) + l0;
+    const int* sj = FWD ? d.fside_j : d.bside_j;
+    const T* dF = (const T*)d.dF;
+    const T* dWv = (const T*)(FWD ? d.dWs : d.dW);
+    auto at = [&](int q) { return FWD ? grec[q].st.pb : grec[q].st.i; };
+    int b = 0, e = 0, en = lv(1), next = t < en ? at(t) : 0;
+    // side slots, a step a level: offsets (level k + 4), cell (k + 3), increments (k + 2), slot (k + 1)
+    const bool side = t < SIDE && staged;
+    int pa = 0, pb = 0, j = -1, jv = -1;
+    T v[13];
+    if (side && nl > 3) { pa = sp[3]; pb = sp[4]; }
+    for (int k = 0; k <= nl; k++) {                                // stores level k - 1
+      if (staged) {
+        if (t == 0) st_release(progress, k);                       // levels below k are finished
+        const int ix = next;
+        if (e + t < en) next = at(e + t);
+        for (int q = b + t; q < e; q += 32 * STORE_WARPS) {
+          const int x = q == b + t ? ix : at(q), slot = q & (S::SLOTS - 1);
+          alignas(16) T w[4];
+          load_co<T>(w, ring + slot * 12 + 8);
+          store_inc<T, FWD>(d, x, w, ring4[slot]);
+        }
+        if (side) {
+          if (jv >= 0) {
+            const int slot = S::SLOTS + ((k + 1) & 1) * SIDE + t;
+#pragma unroll
+            for (int c = 0; c < 12; c++) ring[slot * 12 + c] = v[c];
+            ring4[slot] = v[12];
+          }
+          jv = j;
+          if (jv >= 0) {
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+              v[c] = dF[2 * c * n + jv];
+              v[4 + c] = dF[(2 * c + 1) * n + jv];
+              v[8 + c] = dWv[c * n + jv];
+            }
+            v[12] = dWv[4 * n + jv];
+          }
+          j = pa + t < pb ? sj[pa + t] : -1;
+          if (k + 5 <= nl) { pa = sp[k + 4]; pb = sp[k + 5]; }
+          else pa = pb;
+        }
+      }
+      if (k == nl) break;
+      bar_levels(nct + 32 * STORE_WARPS);
+      b = e; e = en; en = lv(k + 2);
+    }
+  } else if (staged && (tid & 31) == 0) {
+    constexpr int CHUNK = S::CHUNK;
+    const int nchunk = (np + CHUNK - 1) / CHUNK;
+    const unsigned urec = (unsigned)__cvta_generic_to_shared(smem_raw + S::rec);
+    int issued = 0, landed = 0, seen = -1, idle = 0;
+    while (landed < nchunk && idle < d.wait_limit) {
+      const int k = ld_acquire(progress);
+      idle = k == seen ? idle + 1 : 0;
+      if (k != seen) {
+        seen = k;
+        if (k >= nl) break;                                        // the sweep is over
+        const int upto = min(lv(k) / CHUNK + S::NCHUNK, nchunk);
+        // the buffers were read by generic loads: order those before the async proxy's writes
+        if (issued < upto) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        for (; issued < upto; issued++) {
+          if (FWD && d.starve_test && issued == 1) continue;
+          // (a buffer's last chunk, read from global memory where it came late, may be in flight)
+          if (issued - S::NCHUNK >= landed) break;
+          const int c = issued % S::NCHUNK, q = issued * CHUNK, m = min(CHUNK, np - q);
+          const unsigned bytes = (unsigned)(m * sizeof(SweepRec<T>));
+          mbar_expect(bar0 + 8 * c, bytes);
+          bulk_g2s(urec + (unsigned)(c * CHUNK * sizeof(SweepRec<T>)), grec + q, bytes, bar0 + 8 * c);
+        }
+      }
+      if (landed < issued) {
+        if (!mbar_wait(bar0 + 8 * (landed % S::NCHUNK), (unsigned)((landed / S::NCHUNK) & 1), d.wait_limit)) {
+          d.tmo[s] = 1;
+          landed++;                                                // the others in flight land below
+          break;
+        }
+        landed++;
+        st_release(landed_p, landed * CHUNK);
+      } else {
+        __nanosleep(40);
+      }
+    }
+    for (; landed < issued; landed++)                              // let the copies in flight land
+      if (!(FWD && d.starve_test && landed == 1))
+        mbar_wait(bar0 + 8 * (landed % S::NCHUNK), (unsigned)((landed / S::NCHUNK) & 1), d.wait_limit);
+  }
+  if constexpr (FWD) {
+    if constexpr (C == 1) __syncthreads();                         // the increments stored above
+    else cg::this_cluster().sync();
+    ghost_pass<T>(d, s, r * (int)blockDim.x + tid, C * (int)blockDim.x, sa_on);
+  }
 }
 
 template <class T, bool FWD>
-__host__ __device__ constexpr size_t cluster_smem() {
-  return (size_t)13 * RING * sizeof(T) +
-         (size_t)NARROW_THREADS * (sizeof(typename Rec<T, FWD>::Stat) + sizeof(typename Rec<T, FWD>::Dyn));
-}
-
+__global__ void __launch_bounds__(NARROW_THREADS + 32 * (STORE_WARPS + 1), 1)
+k_sweep_block(const __grid_constant__ Dev d) { sweep_narrow<T, FWD, 1>(d); }
 template <class T, bool FWD, int C>
-__device__ __forceinline__ void sweep_cluster(const Dev& d) {
-  using Stat = typename Rec<T, FWD>::Stat;
-  using Dyn = typename Rec<T, FWD>::Dyn;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* ring = (T*)smem_raw;
-  Stat* sst = (Stat*)(smem_raw + (size_t)13 * RING * sizeof(T)) + threadIdx.x;
-  Dyn* sdy = (Dyn*)(smem_raw + (size_t)13 * RING * sizeof(T) + (size_t)NARROW_THREADS * sizeof(Stat)) + threadIdx.x;
-  const int s = d.g_solve0 + blockIdx.x / C, r = blockIdx.x % C;   // one cluster of C blocks per solve
-  if (d.st[s].state != 0 || d.flow[s].scheme == 1) return;         // uniform over the cluster
-  cg::this_cluster().sync();                                       // every block runs before any remote read
-  const bool sa_on = d.flow[s].sa_on;
-  const int* lvl = FWD ? d.fwd_lvl : d.bwd_lvl;
-  const int* lsp = FWD ? d.lvl_solve_ptr : d.blvl_solve_ptr;
-  const int l0 = lsp[s], l1 = lsp[s + 1] - 1;
-  const Stat* gst = FWD ? (const Stat*)d.fst : (const Stat*)d.bst;
-  const Dyn* gdy = (const Dyn*)(FWD ? d.fdyn : d.bdyn);
-  const int pbase = lvl[l0];
-  const int step = C * (int)blockDim.x;
-  int b = lvl[l0], e = lvl[l0 + 1];
-  int pm = first_own<C>(b, pbase, r) + C * (int)threadIdx.x;   // this thread's position of the level
-  if (l0 < l1 && pm < e) { cpa_record(sst, gst + pm); cpa_record(sdy, gdy + pm); cpa_commit(); }
-  for (int l = l0; l < l1; l++) {
-    const int en = (l + 1 < l1) ? lvl[l + 2] : e;
-    const bool mine = pm < e;
-    Stat cs;
-    Dyn cd;
-    if (mine) {
-      cpa_wait_all();
-      cs = load_rec(sst);        // this level's record into registers, freeing the stage
-      cd = load_rec(sdy);
-    }
-    const int pn = first_own<C>(e, pbase, r) + C * (int)threadIdx.x;
-    if (pn < en) { cpa_record(sst, gst + pn); cpa_record(sdy, gdy + pn); cpa_commit(); }
-    if (mine) {
-      if constexpr (FWD) fwd_process<T, C>(d, ring, pm, pbase, cs, cd, sa_on);
-      else bwd_process<T, C>(d, ring, pm, pbase, cs, cd, sa_on);
-    }
-    for (int p = pm + step; p < e; p += step) {   // levels wider than the cluster's threads
-      const Stat xs = load_rec(gst + p);
-      const Dyn xd = load_rec(gdy + p);
-      if constexpr (FWD) fwd_process<T, C>(d, ring, p, pbase, xs, xd, sa_on);
-      else bwd_process<T, C>(d, ring, p, pbase, xs, xd, sa_on);
-    }
-    cg::this_cluster().sync();   // release/acquire over the cluster's shared and global writes
-    b = e;
-    e = en;
-    pm = pn;
-  }
-}
-
-template <class T, int C>
-__global__ void __launch_bounds__(NARROW_THREADS) k_sweep_fwd_cluster(Dev d) { sweep_cluster<T, true, C>(d); }
-template <class T, int C>
-__global__ void __launch_bounds__(NARROW_THREADS) k_sweep_bwd_cluster(Dev d) { sweep_cluster<T, false, C>(d); }
+__global__ void __launch_bounds__(NARROW_THREADS) k_sweep_cluster(const __grid_constant__ Dev d) { sweep_narrow<T, FWD, C>(d); }
 
 // ---- wide schedule: one launch per level, all solves ----
 template <class T>
@@ -908,32 +1123,32 @@ void launch_update(const Dev& d, int precision, cudaStream_t s) {
   else k_update<double><<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
 }
 
-template <class T>
+template <class T, bool FWD>
 static void set_smem_t() {
-  cudaFuncSetAttribute(k_sweep_fwd_bulk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bulk_smem<T, true>());
-  cudaFuncSetAttribute(k_sweep_bwd_bulk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bulk_smem<T, false>());
-  cudaFuncSetAttribute(k_sweep_fwd_cluster<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem<T, true>());
-  cudaFuncSetAttribute(k_sweep_bwd_cluster<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem<T, false>());
-  cudaFuncSetAttribute(k_sweep_fwd_cluster<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem<T, true>());
-  cudaFuncSetAttribute(k_sweep_bwd_cluster<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem<T, false>());
-  cudaFuncSetAttribute(k_sweep_fwd_cluster<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem<T, true>());
-  cudaFuncSetAttribute(k_sweep_bwd_cluster<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem<T, false>());
+  const int bytes = (int)Smem<T>::total;
+  cudaFuncSetAttribute(k_sweep_block<T, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaFuncSetAttribute(k_sweep_cluster<T, FWD, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaFuncSetAttribute(k_sweep_cluster<T, FWD, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaFuncSetAttribute(k_sweep_cluster<T, FWD, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 void setup_sweeps() {
-  set_smem_t<double>();
-  set_smem_t<float>();
-  set_smem_t<df64>();
+  set_smem_t<double, true>();
+  set_smem_t<double, false>();
+  set_smem_t<float, true>();
+  set_smem_t<float, false>();
+  set_smem_t<df64, true>();
+  set_smem_t<df64, false>();
 }
 
 // one cluster of C blocks per solve
-template <class T, int C>
-static void launch_cluster(bool fwd, const Dev& d, int threads, cudaStream_t s) {
-  void (*k)(Dev) = fwd ? k_sweep_fwd_cluster<T, C> : k_sweep_bwd_cluster<T, C>;
+template <class T, bool FWD, int C>
+static void launch_cluster(const Dev& d, int threads, cudaStream_t s) {
+  void (*k)(Dev) = k_sweep_cluster<T, FWD, C>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(d.g_nsolve * C));
   cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = fwd ? cluster_smem<T, true>() : cluster_smem<T, false>();
+  cfg.dynamicSmemBytes = Smem<T>::total;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -945,15 +1160,14 @@ static void launch_cluster(bool fwd, const Dev& d, int threads, cudaStream_t s) 
   cudaLaunchKernelEx(&cfg, k, d);
 }
 
-template <class T>
-static void launch_narrow_c(bool fwd, const Dev& d, int threads, cudaStream_t s) {
+template <class T, bool FWD>
+static void launch_narrow(const Dev& d, int threads, cudaStream_t s) {
   switch (d.sweep_cluster) {
-    case 2: launch_cluster<T, 2>(fwd, d, threads, s); break;
-    case 4: launch_cluster<T, 4>(fwd, d, threads, s); break;
-    case 8: launch_cluster<T, 8>(fwd, d, threads, s); break;
-    default:   // one block per solve
-      if (fwd) k_sweep_fwd_bulk<T><<<d.g_nsolve, threads, bulk_smem<T, true>(), s>>>(d);
-      else k_sweep_bwd_bulk<T><<<d.g_nsolve, threads, bulk_smem<T, false>(), s>>>(d);
+    case 2: launch_cluster<T, FWD, 2>(d, threads, s); break;
+    case 4: launch_cluster<T, FWD, 4>(d, threads, s); break;
+    case 8: launch_cluster<T, FWD, 8>(d, threads, s); break;
+    default:   // one block per solve: the cells' threads, the store warps and the copy warp
+      k_sweep_block<T, FWD><<<d.g_nsolve, threads + 32 * (STORE_WARPS + 1), Smem<T>::total, s>>>(d);
       break;
   }
 }
@@ -975,9 +1189,9 @@ void launch_sweep_fwd(const Dev& d, int precision, int threads, cudaStream_t s) 
     }
     return;
   }
-  if (precision == 1) launch_narrow_c<float>(true, d, threads, s);
-  else if (precision == 2) launch_narrow_c<df64>(true, d, threads, s);
-  else launch_narrow_c<double>(true, d, threads, s);
+  if (precision == 1) launch_narrow<float, true>(d, threads, s);
+  else if (precision == 2) launch_narrow<df64, true>(d, threads, s);
+  else launch_narrow<double, true>(d, threads, s);
 }
 
 void launch_sweep_bwd(const Dev& d, int precision, int threads, cudaStream_t s) {
@@ -991,9 +1205,9 @@ void launch_sweep_bwd(const Dev& d, int precision, int threads, cudaStream_t s) 
     }
     return;
   }
-  if (precision == 1) launch_narrow_c<float>(false, d, threads, s);
-  else if (precision == 2) launch_narrow_c<df64>(false, d, threads, s);
-  else launch_narrow_c<double>(false, d, threads, s);
+  if (precision == 1) launch_narrow<float, false>(d, threads, s);
+  else if (precision == 2) launch_narrow<df64, false>(d, threads, s);
+  else launch_narrow<double, false>(d, threads, s);
 }
 
 }  // namespace igks
