@@ -130,6 +130,8 @@ static DevFlow make_devflow(const igks_flow& f) {
   d.res_target = f.res_target; d.venkat_k = f.venkat_k; d.c_num = f.c_num;
   d.eq40_target = f.eq40_target;
   d.pr_fix = 1.0 / f.prandtl - 1.0;
+  d.tr_h = 2.0 * d.lam_inf;
+  d.visc_c = d.mu_inf * (1.0 + d.s_star) * d.tr_h * std::sqrt(d.tr_h);
   d.sa_on = f.sa_on; d.limiter = f.limiter; d.visc_sr = f.visc_sr; d.scheme = f.scheme;
   return d;
 }
@@ -208,7 +210,7 @@ static void enqueue_iteration(igks_ctx* ctx, int g) {
   launch_prep(d, s);                   if (t) cudaEventRecordWithFlags(ev[e++], s, cudaEventRecordExternal);
   launch_ghost(d, s);                  if (t) cudaEventRecordWithFlags(ev[e++], s, cudaEventRecordExternal);
   launch_gradient(d, s);               if (t) cudaEventRecordWithFlags(ev[e++], s, cudaEventRecordExternal);
-  launch_flux(d, s);                   if (t) cudaEventRecordWithFlags(ev[e++], s, cudaEventRecordExternal);
+  launch_flux(d, p, s);                 if (t) cudaEventRecordWithFlags(ev[e++], s, cudaEventRecordExternal);
   launch_residual(d, s);               if (t) cudaEventRecordWithFlags(ev[e++], s, cudaEventRecordExternal);
   launch_norms(d, s);                  if (t) cudaEventRecordWithFlags(ev[e++], s, cudaEventRecordExternal);
   launch_sweep_prep(d, p, s);          if (t) cudaEventRecordWithFlags(ev[e++], s, cudaEventRecordExternal);
@@ -596,7 +598,7 @@ static int build(igks_ctx* ctx) {
   AL(W, double, 5 * (size_t)nc); AL(grad, double, 8 * (size_t)nc); AL(phi, double, 4 * (size_t)nc);
   AL(omega, double, nc); AL(mu_l, double, nc); AL(mu_t, double, nc); AL(Lam, double, nc);
   AL(pu, double, nc); AL(pv, double, nc); AL(pc, double, nc); AL(lsq, double, 4 * (size_t)nc);
-  AL(M, double, 5 * (size_t)nc); AL(fw, double, nc); AL(sa_diag, double, nc);
+  AL(M, double, 5 * (size_t)nc); AL(nul, double, nc); AL(sa_diag, double, nc);
   AL(dWs, double, 5 * (size_t)nc); AL(dW, double, 5 * (size_t)nc); AL(dF, double, 8 * (size_t)nc);
   AL(fS, double, nf); AL(fnx, double, nf); AL(fny, double, nf); AL(fmx, double, nf); AL(fmy, double, nf);
   AL(fcx, double, nf); AL(fcy, double, nf); AL(fidL, double, nf); AL(fidR, double, nf); AL(fdn, double, nf);
@@ -609,7 +611,7 @@ static int build(igks_ctx* ctx) {
   d.wait_limit = ctx->opt.wait_limit > 0 ? ctx->opt.wait_limit : DEFAULT_WAIT_LIMIT;
   d.starve_test = ctx->opt.starve_test;
   d.nnz = (int)cf_face.size();
-  AL(sw_cell, double, 5 * (size_t)nc); AL(sw_st, double, 4 * (size_t)d.nnz); AL(sw_j, int, d.nnz);
+  AL(sw_cell, double, 5 * (size_t)nc); AL(sw_st, double, std::max(4 * (size_t)d.nnz, 8 * (size_t)nc)); AL(sw_j, int, d.nnz);
   UP(fs_ptr, fs_ptr); UP(fs_j, fs_j); UP(fs_slot, fs_slot); UP(cf_to_fs, cf_to_fs);
   UP(bs_ptr, bs_ptr); UP(bs_j, bs_j); UP(bs_slot, bs_slot); UP(cf_to_bs, cf_to_bs);
   d.nfs = (int)fs_j.size();
@@ -628,7 +630,9 @@ static int build(igks_ctx* ctx) {
   UP(gent_ptr, gent_ptr); UP(gent_pos, gent_pos);
   d.ring = ring;
   AL(gprim, double, 6 * (size_t)nf);
+  d.lgrad = (double*)d.sw_st;
   setup_sweeps();
+  CK(flux_table_init());
   {
     // wide schedule: level l of every solve, solves in order
     int maxf = 0, maxb = 0;

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_prep(Dev d) {
   const double h = p * ir;
   const double mu = viscosity_h(fl, h);
   d.mu_l[i] = mu;
+  d.nul[i] = mu * ir;
   double mt = 0.0;
   if (fl.sa_on && nut > 0.0) {   // mu_t = rho nu~ fv1 (Eq. 34)
     const double chi = nut * r * __drcp_rn(mu), c3 = chi * chi * chi;
@@ -323,6 +324,12 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
     }
 #pragma unroll
     for (int v = 0; v < 4; v++) d.phi[v * n + i] = phi[v];
+    if (fl.limiter)   // limited once per cell for the three or four faces that read it
+#pragma unroll
+      for (int v = 0; v < 4; v++) {
+        d.lgrad[(2 * v) * n + i] = phi[v] * b[2 * v];
+        d.lgrad[(2 * v + 1) * n + i] = phi[v] * b[2 * v + 1];
+      }
     const double ir = __drcp_rn(Wi[0]);
     double u = Wi[1] * ir, vv = Wi[2] * ir;
     double dudy = (b[3] - u * b[1]) * ir;
@@ -384,7 +391,7 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_residual(Dev d) {
     for (int v = 0; v < 4; v++) d.M[v * n + i] = -acc[v] * idt;
     double area = d.area[i];
     const double iarea = __drcp_rn(area);
-    double m4 = 0.0, fw = 0.0, sdiag = 0.0;
+    double m4 = 0.0, sdiag = 0.0;
     if (fl.sa_on) {
       // Eq. 28a with SA-noft2 and the 2012 clipping of S~; the wall distance enters through
       // 1/d, the viscosity ratio through chi = nu~ rho / mu, and x^(1/6) is cbrt(sqrt(x))
@@ -404,14 +411,13 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_residual(Dev d) {
       double g = rr + SA_CW2 * (r6 - rr);
       double g2 = g * g, g6 = g2 * g2 * g2;
       const double c6 = SA_CW3 * SA_CW3 * SA_CW3 * SA_CW3 * SA_CW3 * SA_CW3;
-      fw = g * cbrt(sqrt((1.0 + c6) * __drcp_rn(g6 + c6)));
+      const double fw = g * cbrt(sqrt((1.0 + c6) * __drcp_rn(g6 + c6)));
       double nd = nut * idw;
       double Sr = SA_CB1 * St * nut - SA_CW1 * fw * nd * nd;
       m4 = area * Sr + acc[4];
       sdiag = sad + area * 2.0 * SA_CW1 * fw * nut * idw * idw;
     }
     d.M[4 * n + i] = m4;
-    d.fw[i] = fw;
     d.sa_diag[i] = sdiag;
     double mr = d.M[i];
     rmax = fabs(mr);

@@ -27,6 +27,7 @@ struct DevFlow {
   double Winf[5];
   double cfl_exp, cfl_init, cfl_min, cfl_max, res_target, venkat_k, c_num, eq40_target;
   double pr_fix;   // 1/Pr - 1, the factor of the Prandtl-number fix
+  double tr_h, visc_c;   // T/T_inf = tr_h h; Sutherland: mu = visc_c h^(3/2) / (tr_h h + s_star)
   int sa_on, limiter, visc_sr, scheme;
 };
 
@@ -101,7 +102,9 @@ struct Dev {
   double* lsq;              // [4][nc_pad] least-squares normal matrix A00, A01, A11 and 1/det (geometry)
   double* Lam;              // [nc_pad] sum over faces of (Lambda_c)_ij
   double* M;                // [5][nc_pad]
-  double* fw;               // [nc_pad]
+  double* nul;              // [nc_pad] laminar kinematic viscosity (k_prep)
+  double* lgrad;            // [8][nc_pad] limited gradients of solves with a limiter, from k_gradient
+                            // to k_flux (the memory of sw_st, which the pre-pass writes later)
   double* sa_diag;          // [nc_pad] SA diagonal without the Omega/dt_imp term
   void* dWs;                // [5][nc_pad] of T (sweep type)
   void* dW;                 // [5][nc_pad] of T
@@ -189,7 +192,8 @@ void launch_init_state(const Dev& d, int solve, cudaStream_t s);
 void launch_prep(const Dev& d, cudaStream_t s);
 void launch_ghost(const Dev& d, cudaStream_t s);
 void launch_gradient(const Dev& d, cudaStream_t s);
-void launch_flux(const Dev& d, cudaStream_t s);
+cudaError_t flux_table_init();   // the flux's device table, once per device (current device)
+void launch_flux(const Dev& d, int precision, cudaStream_t s);
 void launch_residual(const Dev& d, cudaStream_t s);
 void launch_norms(const Dev& d, cudaStream_t s);
 void setup_sweeps();   // kernel attributes (shared-memory ring size), once per build
