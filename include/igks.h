@@ -297,8 +297,8 @@ int igks_destroy(igks_ctx* ctx);
  *   stream cudaStream_t the two kernels run on (NULL: the legacy default stream)
  * It computes the same reduction, in the same order, as igks_iterate does for its
  * status. Inputs and outputs belong to the caller; the only other memory used is a
- * fixed scratch array in the library's device data (IGKS_NOALLOC_MAX_CELLS / 256 * 2
- * doubles = 64 KiB, held on every GPU that loads the library until the process exits).
+ * fixed scratch array in the library's device data (IGKS_NOALLOC_MAX_CELLS / 64 * 2
+ * doubles = 256 KiB, held on every GPU that loads the library until the process exits).
  * Its device address is looked up once per device, with that device current, by the
  * first call made on that device: make that first call before any stream capture.
  * Every call shares the scratch array and it keeps the last call's contents; each call

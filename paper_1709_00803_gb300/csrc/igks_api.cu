@@ -518,7 +518,7 @@ static int build(igks_ctx* ctx) {
     std::memset(&q, 0, sizeof q);
     q.cfl = ctx->flows[s].cfl_init;
     q.blk_begin = co / CELL_BLOCK;
-    q.blk_end = (co + ctx->cell_pad[s]) / CELL_BLOCK;
+    q.blk_end = (co + m.nc + CELL_BLOCK - 1) / CELL_BLOCK;
     q.cell_begin = co;
     q.cell_end = co + m.nc;
     dfl[s] = make_devflow(ctx->flows[s]);

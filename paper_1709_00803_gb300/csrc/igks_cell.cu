@@ -137,6 +137,27 @@ __device__ __forceinline__ bool cell_live(const Dev& d, int i, int* solve) {
   return true;
 }
 
+// Comparisons of doubles as integers: an FP64 maximum costs a slot of the FP64 pipe, as much
+// as a multiply-add, integer instructions are all but free beside it. ord_of: an
+// order-preserving map to signed integers; bits_of: the bits, ordered like the values for
+// non-negative doubles.
+__device__ __forceinline__ long long ord_of(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double of_ord(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+__device__ __forceinline__ unsigned long long bits_of(double x) { return (unsigned long long)__double_as_longlong(x); }
+__device__ __forceinline__ double of_bits(unsigned long long k) { return __longlong_as_double((long long)k); }
+// warp minimum / maximum of 64-bit patterns: high words, then the low words of the extreme one
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long x) {
+  const unsigned hi = (unsigned)(x >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? (unsigned)x : 0xffffffffu);
+  return ((unsigned long long)mh << 32) | ml;
+}
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long x) { return ~warp_min(~x); }
+
 // velocity and sound speed of a state, in the order the face spectral radius uses them
 __device__ __forceinline__ void speeds_of(const double* W, double* u, double* v, double* c) {
   const double p = pressure_of(W[0], W[1], W[2], W[3]);
@@ -241,15 +262,18 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
   const int blk = d.g_blk0 + blockIdx.x;
   int i = blk * CELL_BLOCK + threadIdx.x, s = -1;
   bool live = cell_live(d, i, &s);
-  double dtc = DBL_MAX;
+  unsigned long long dtc = ~0ull;   // bits of the cell's time step
   if (live) {
     const DevFlow& fl = d.flow[s];
     const int n = d.nc_pad;
     double Wi[5];
     for (int v = 0; v < 5; v++) Wi[v] = d.W[v * n + i];
     double xi = d.cx[i], yi = d.cy[i];
-    double r0[4] = {0, 0, 0, 0}, r1[4] = {0, 0, 0, 0}, wmax[4], wmin[4];
-    for (int v = 0; v < 4; v++) wmax[v] = wmin[v] = Wi[v];
+    const bool lim = fl.limiter != 0;
+    double r0[4] = {0, 0, 0, 0}, r1[4] = {0, 0, 0, 0};
+    long long kmax[4], kmin[4];       // extremes over the cell and its neighbours (ord_of)
+#pragma unroll
+    for (int v = 0; v < 4; v++) kmax[v] = kmin[v] = ord_of(Wi[v]);
     double Lam = 0.0;
     for (int k = d.cf_ptr[i]; k < d.cf_ptr[i + 1]; k++) {
       int f = d.cf_face[k];
@@ -264,11 +288,17 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
         double dw = Wk[v] - Wi[v];
         r0[v] += dx * dw;
         r1[v] += dy * dw;
-        wmax[v] = fmax(wmax[v], Wk[v]);
-        wmin[v] = fmin(wmin[v], Wk[v]);
       }
-      Lam += 0.5 * d.lam_f[f] * d.fS[f];
+      if (lim)
+#pragma unroll
+        for (int v = 0; v < 4; v++) {
+          const long long k_ = ord_of(Wk[v]);
+          kmax[v] = max(kmax[v], k_);
+          kmin[v] = min(kmin[v], k_);
+        }
+      Lam += d.lam_f[f] * d.fS[f];
     }
+    Lam *= 0.5;   // (exact: the bits of summing halves)
     // the geometry's normal matrix and 1/det (k_lsq_matrix)
     const double A00 = d.lsq[i], A01 = d.lsq[n + i], A11 = d.lsq[2 * n + i], idet = d.lsq[3 * n + i];
     double area = d.area[i];
@@ -286,39 +316,47 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
       // excursion of each sign (correctly rounded division is monotone in the divisor),
       // so two divisions per variable give the same bits as one per vertex; and a
       // correctly rounded x / y with 0 < x < y stays below 1, so min(1, x / y) is 1
-      // exactly when x >= y and the division is needed only where the limiter acts
-      double up[4] = {0, 0, 0, 0}, dn[4] = {0, 0, 0, 0};
+      // exactly when x >= y and the division is needed only where the limiter acts.
+      // Magnitudes of one sign are compared by their bits.
+      unsigned long long up[4] = {0, 0, 0, 0}, dn[4] = {0, 0, 0, 0};
       for (int k = d.cn_ptr[i]; k < d.cn_ptr[i + 1]; k++) {
         int nd = d.cn_node[k];
         double ox = d.xy[nd] - xi, oy = d.xy[d.nn + nd] - yi;
 #pragma unroll
         for (int v = 0; v < 4; v++) {
-          double dv = b[2 * v] * ox + b[2 * v + 1] * oy;
-          up[v] = fmax(up[v], dv);
-          dn[v] = fmin(dn[v], dv);
+          const unsigned long long q = bits_of(b[2 * v] * ox + b[2 * v + 1] * oy);
+          const unsigned long long m = q & 0x7fffffffffffffffull;
+          if (q == m) up[v] = max(up[v], m);
+          else dn[v] = max(dn[v], m);
         }
       }
 #pragma unroll
       for (int v = 0; v < 4; v++) {
-        const double hi = wmax[v] - Wi[v], lo = wmin[v] - Wi[v];
-        if (up[v] > 0.0 && hi < up[v]) phi[v] = fmin(phi[v], hi / up[v]);
-        if (dn[v] < 0.0 && lo > dn[v]) phi[v] = fmin(phi[v], lo / dn[v]);
+        const double hi = of_ord(kmax[v]) - Wi[v], lo = Wi[v] - of_ord(kmin[v]);
+        if (bits_of(hi) < up[v]) phi[v] = hi / of_bits(up[v]);
+        if (bits_of(lo) < dn[v]) {
+          const double q = lo / of_bits(dn[v]);
+          if (bits_of(q) < bits_of(phi[v])) phi[v] = q;
+        }
       }
     } else if (fl.limiter == 2) {
       double h = sqrt(area);
       double eps2 = (fl.venkat_k * h) * (fl.venkat_k * h) * (fl.venkat_k * h);
+      double hi[4], lo[4];
+#pragma unroll
+      for (int v = 0; v < 4; v++) { hi[v] = of_ord(kmax[v]) - Wi[v]; lo[v] = of_ord(kmin[v]) - Wi[v]; }
       for (int k = d.cn_ptr[i]; k < d.cn_ptr[i + 1]; k++) {
         int nd = d.cn_node[k];
         double ox = d.xy[nd] - xi, oy = d.xy[d.nn + nd] - yi;
 #pragma unroll
         for (int v = 0; v < 4; v++) {
           double dv = b[2 * v] * ox + b[2 * v + 1] * oy;
-          double pv = 1.0;
-          if (dv != 0.0) {
-            double dp = dv > 0.0 ? wmax[v] - Wi[v] : wmin[v] - Wi[v];
-            pv = ((dp * dp + eps2) * dv + 2.0 * dv * dv * dp) / (dv * (dp * dp + 2.0 * dv * dv + dv * dp + eps2));
+          if (bits_of(dv) << 1) {   // not zero
+            const double dp = __double2hiint(dv) < 0 ? lo[v] : hi[v];
+            const double a = dp * dp, c = 2.0 * dv * dv;
+            const double pv = ((a + eps2) * dv + c * dp) / (dv * (a + c + dv * dp + eps2));
+            if (ord_of(pv) < ord_of(phi[v])) phi[v] = pv;
           }
-          phi[v] = fmin(phi[v], pv);
         }
       }
     }
@@ -336,23 +374,12 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
     double dvdx = (b[4] - vv * b[0]) * ir;
     d.omega[i] = fabs(dvdx - dudy);
     d.Lam[i] = Lam;
-    dtc = fl.cfl_exp * area / Lam;
+    dtc = bits_of(fl.cfl_exp * area / Lam);   // positive doubles order like their bits
   }
-  // block minimum -> one atomic per block; every block lies inside one solve
-  __shared__ double red[CELL_BLOCK / 32];
-  double m = dtc;
-  for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    m = threadIdx.x < CELL_BLOCK / 32 ? red[threadIdx.x] : DBL_MAX;
-    for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (threadIdx.x == 0 && m < DBL_MAX) {
-      int bs = d.cell_solve[blk * CELL_BLOCK];
-      // positive doubles order like their bit patterns
-      if (bs >= 0) atomicMin(d.dt_bits + bs, (unsigned long long)__double_as_longlong(m));
-    }
-  }
+  // warp minimum -> at most one atomic per warp; every block lies inside one solve
+  dtc = warp_min(dtc);
+  if ((threadIdx.x & 31) == 0 && live && dtc < *(volatile unsigned long long*)(d.dt_bits + s))
+    atomicMin(d.dt_bits + s, dtc);
 }
 
 void launch_gradient(const Dev& d, cudaStream_t s) {
@@ -424,17 +451,17 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_residual(Dev d) {
     double q = mr * iarea;
     r2 = q * q;
   }
-  __shared__ double smax[CELL_BLOCK / 32], ssum[CELL_BLOCK / 32];
-  for (int o = 16; o > 0; o >>= 1) {
-    rmax = fmax(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-    r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-  }
-  if ((threadIdx.x & 31) == 0) { smax[threadIdx.x >> 5] = rmax; ssum[threadIdx.x >> 5] = r2; }
+  __shared__ double ssum[CELL_BLOCK / 32];
+  __shared__ unsigned long long smax[CELL_BLOCK / 32];
+  const unsigned long long wm = warp_max(bits_of(rmax));
+  for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
+  if ((threadIdx.x & 31) == 0) { smax[threadIdx.x >> 5] = wm; ssum[threadIdx.x >> 5] = r2; }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int w = 0; w < CELL_BLOCK / 32; w++) { a = fmax(a, smax[w]); b += ssum[w]; }
-    d.part[blk] = a;
+    unsigned long long a = 0;
+    double b = 0.0;
+    for (int w = 0; w < CELL_BLOCK / 32; w++) { a = max(a, smax[w]); b += ssum[w]; }
+    d.part[blk] = of_bits(a);
     d.part[d.n_cell_blocks + blk] = b;
   }
 }
@@ -443,18 +470,17 @@ void launch_residual(const Dev& d, cudaStream_t s) {
   k_residual<<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
 }
 
-// per-solve norms in fixed block order, CFL adaptation (Eq. 25), stopping rule
-__global__ void k_norms(Dev d) {
-  int s = d.g_solve0 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= d.g_solve0 + d.g_nsolve) return;
+// per-solve norms, CFL adaptation (Eq. 25), stopping rule; one block per solve, the blocks'
+// partial norms added in a fixed order (thread t takes blocks t, t + NORM_THREADS, ..., then
+// a tree): one thread walking 235 blocks took 36 us.
+__global__ void __launch_bounds__(NORM_THREADS) k_norms(Dev d) {
+  const int s = d.g_solve0 + blockIdx.x;
   SolveState& st = d.st[s];
   if (st.state != 0) return;
   const DevFlow& fl = d.flow[s];
-  double rmax = 0.0, r2 = 0.0;
-  for (int b = st.blk_begin; b < st.blk_end; b++) {
-    rmax = fmax(rmax, d.part[b]);
-    r2 += d.part[d.n_cell_blocks + b];
-  }
+  double rmax, r2;
+  norm_reduce(d.part + st.blk_begin, d.part + d.n_cell_blocks + st.blk_begin, st.blk_end - st.blk_begin, &rmax, &r2);
+  if (threadIdx.x != 0) return;
   st.dt = __longlong_as_double((long long)d.dt_bits[s]);
   st.res_inf = rmax;
   st.res_l2 = sqrt(r2 / (double)(st.cell_end - st.cell_begin));
@@ -472,6 +498,7 @@ __global__ void k_norms(Dev d) {
     else c = (st.res_inf_prev > 0.0) ? fl.cfl_max : st.cfl;
     st.cfl = fmin(fmax(c, fl.cfl_min), fl.cfl_max);
   }
+  st.icfl = __drcp_rn(st.cfl);
   st.res_inf_prev = st.res_inf;
   // converged at res_target times the first residual; an exactly zero residual (also at the
   // first iteration) has nothing left to fall
@@ -479,7 +506,7 @@ __global__ void k_norms(Dev d) {
 }
 
 void launch_norms(const Dev& d, cudaStream_t s) {
-  k_norms<<<(d.g_nsolve + 63) / 64, 64, 0, s>>>(d);
+  k_norms<<<d.g_nsolve, NORM_THREADS, 0, s>>>(d);
 }
 
 __global__ void k_end_iter(Dev d) {
@@ -487,7 +514,7 @@ __global__ void k_end_iter(Dev d) {
   if (s >= d.g_solve0 + d.g_nsolve) return;
   SolveState& st = d.st[s];
   if (st.state != 0) return;
-  st.eq40 = __longlong_as_double((long long)d.eq40_bits[s]);
+  st.eq40 = sqrt(__longlong_as_double((long long)d.eq40_bits[s]));   // k_update keeps the squares
   const double e40 = d.flow[s].eq40_target;
   if (st.pending == 0 && e40 > 0.0 && st.eq40 <= e40) st.pending = 1;   // Eq. 40 criterion
   if (d.bad[s]) st.pending = -5;   // IGKS_DIVERGED

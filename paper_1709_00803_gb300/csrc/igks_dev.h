@@ -10,12 +10,18 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "igks_norm.cuh"
+
 namespace igks {
 
 constexpr int KDOF = 3;                                  // internal degrees of freedom (Eq. 2)
 constexpr double GAMMA = (KDOF + 4.0) / (KDOF + 2.0);    // 1.4
 constexpr int CELL_ALIGN = 256;
-constexpr int CELL_BLOCK = 256;                          // block of the per-cell kernels
+// Block of the per-cell kernels: they are bound by the FP64 pipe of an SM, so a small mesh
+// wants its cells on as many SMs as it has warps for (20,480 cells: 80 blocks of 256 threads
+// left half of the 152 SMs idle; 64 threads make 320). Large meshes do not care.
+constexpr int CELL_BLOCK = 64;
+static_assert(CELL_BLOCK == NORM_CELLS, "a block of the residual kernel gives one partial norm");
 
 // Spalart-Allmaras (SA-noft2 with the 2012 S-tilde clipping)
 constexpr double SA_CB1 = 0.1355, SA_CB2 = 0.622, SA_SIGMA = 2.0 / 3.0, SA_KAPPA = 0.41;
@@ -70,11 +76,12 @@ static_assert(sizeof(SweepStat) == 32 && sizeof(SweepJ) == 16, "static record si
 static_assert(sizeof(SweepRec<float>) == 160 && sizeof(SweepRec<double>) == 288, "record size");
 
 struct SolveState {
+  double icfl;    // 1 / cfl
   double dt, cfl, res_inf, res_l2, res_l2_first, res_inf_prev, eq40;
   int iter;
   int state;      // 0 running, 1 converged, <0 error; read by every kernel of an iteration
   int pending;    // state to take at the end of the current iteration
-  int blk_begin, blk_end;      // per-cell-kernel blocks of this solve
+  int blk_begin, blk_end;      // per-cell-kernel blocks of this solve that hold cells
   int cell_begin, cell_end;    // [begin, end) real cells
 };
 

@@ -55,7 +55,7 @@ __device__ __forceinline__ void side_of(const Dev& d, const double* gr, int c, d
   rot(st, nx, ny, St);
 }
 
-__global__ void __launch_bounds__(128) k_flux(Dev d) {
+__global__ void __launch_bounds__(128, 1) k_flux(Dev d) {
   const int f = d.g_face0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= d.g_face0 + d.g_nface) return;
   const int s = d.fsolve[f];
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(128) k_flux(Dev d) {
   d.sa_a[3 * nf + f] = dgr;
 }
 
-__global__ void __launch_bounds__(128) k_flux_moment(Dev d) {
+__global__ void __launch_bounds__(128, 1) k_flux_moment(Dev d) {
   const int f = d.g_face0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= d.g_face0 + d.g_nface) return;
   const int s = d.fsolve[f];

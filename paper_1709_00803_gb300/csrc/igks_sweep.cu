@@ -211,13 +211,12 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_sweep_prep(Dev d) {
   if (s < 0 || d.st[s].state != 0 || d.flow[s].scheme == 1) return;   // explicit solves: no sweeps
   const DevFlow& fl = d.flow[s];
   const int n = d.nc_pad, nf = d.nf;
-  const double cfl = d.st[s].cfl;
   const double Lam = d.Lam[i];
   const double r = d.W[i], mx = d.W[n + i], my = d.W[2 * n + i], E = d.W[3 * n + i];
   const double u = d.pu[i], v = d.pv[i];          // mx / r, my / r (k_prep)
   const double p = (GAMMA - 1.0) * (E - 0.5 * (mx * u + my * v));
   T cc[5];
-  const double lc = Lam * __drcp_rn(cfl);                                 // Omega / dt_imp (Eq. 24)
+  const double lc = Lam * d.st[s].icfl;                                 // Omega / dt_imp (Eq. 24)
   cc[0] = (T)__drcp_rn(lc + Lam);                                        // 1/D (Eq. 20)
   cc[1] = fl.sa_on ? (T)__drcp_rn(lc + d.sa_diag[i]) : (T)0;             // 1/a_ii (Eq. 32)
   cc[2] = (T)u;
@@ -441,7 +440,7 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_update(Dev d) {
   const int blk = d.g_blk0 + blockIdx.x;
   const int i = blk * CELL_BLOCK + threadIdx.x;
   const int s = d.cell_solve[blk * CELL_BLOCK];   // every block lies in one solve
-  double eq40 = 0.0;
+  double eq40 = 0.0;                              // squared Eq. 40 ratio (the root once per solve)
   int bad = 0;
   // a solve whose sweep wait ran out keeps its state (the increments are incomplete)
   const bool live = (i < d.nc_pad) && d.cell_solve[i] >= 0 && d.st[d.cell_solve[i]].state == 0 &&
@@ -466,8 +465,8 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_update(Dev d) {
     }
     Wi[4] += expl ? (d.flow[si].sa_on ? xf * d.M[4 * n + i] : 0.0) : to_double(dWo[4 * n + i]);
     if (Wi[4] < 0.0) Wi[4] = 0.0;
-    eq40 = sqrt(num) / sqrt(den);
-    const double p = pressure_of(Wi[0], Wi[1], Wi[2], Wi[3]);
+    eq40 = num * __drcp_rn(den);
+    const double p = Wi[3] - 0.5 * (Wi[1] * Wi[1] + Wi[2] * Wi[2]) * __drcp_rn(Wi[0]);   // for its sign
     if (!(Wi[0] > 0.0) || !(p > 0.0) || !isfinite(Wi[3]) || !isfinite(Wi[4])) bad = 1;
 #pragma unroll
     for (int v = 0; v < 5; v++) d.W[v * n + i] = Wi[v];
@@ -475,25 +474,18 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_update(Dev d) {
   flush_eq40(d, (s >= 0 && d.st[s].state == 0) ? s : -1, eq40, bad);
 }
 
-// block-wide max of the Eq. 40 ratio and OR of the divergence flag, one atomic each;
+// warp maximum of the squared Eq. 40 ratio and OR of the divergence flag, one atomic each;
 // positive doubles order like their bit patterns, so the per-solve maximum is exact
 __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int bad) {
-  __shared__ double sm[32];
-  __shared__ int sb[32];
-  for (int o = 16; o > 0; o >>= 1) {
-    eq40 = fmax(eq40, __shfl_xor_sync(0xffffffffu, eq40, o));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-  }
-  if ((threadIdx.x & 31) == 0) { sm[threadIdx.x >> 5] = eq40; sb[threadIdx.x >> 5] = bad; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0;
-    int b = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) { a = fmax(a, sm[w]); b |= sb[w]; }
-    if (s >= 0) {
-      if (a > 0.0) atomicMax(d.eq40_bits + s, (unsigned long long)__double_as_longlong(a));
-      if (b) atomicOr(d.bad + s, 1);
-    }
+  // (a ratio that is not a number comes with bad; it must not pass for a large one)
+  const unsigned long long x = eq40 > 0.0 ? (unsigned long long)__double_as_longlong(eq40) : 0ull;
+  const unsigned hi = (unsigned)(x >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)x : 0u);
+  bad = __any_sync(0xffffffffu, bad);
+  if ((threadIdx.x & 31) == 0 && s >= 0) {
+    const unsigned long long a = ((unsigned long long)mh << 32) | ml;
+    if (a > *(volatile unsigned long long*)(d.eq40_bits + s)) atomicMax(d.eq40_bits + s, a);
+    if (bad) atomicOr(d.bad + s, 1);
   }
 }
 
