@@ -296,7 +296,10 @@ cudaError_t flux_table_init() {
 }
 
 void launch_flux(const Dev& d, int precision, cudaStream_t s) {
-  const int b = d.flux_block > 0 ? d.flux_block : 128;
+  // one-warp blocks by default: the FP64 pipe is shared by an SM, and whole warps spread a small
+  // mesh over the SMs most evenly (20,200 faces: 55 us with blocks of 128, 43 with 32; the same from
+  // 35,000 faces on)
+  const int b = d.flux_block > 0 ? d.flux_block : 32;
   if (!d.g_nface) return;
   if (precision == 1) k_flux_moment<<<(d.g_nface + b - 1) / b, b, 0, s>>>(d);
   else k_flux<<<(d.g_nface + b - 1) / b, b, 0, s>>>(d);
