@@ -21,6 +21,8 @@ using namespace igks;
 // last error of the context-free entry point (igks_noalloc.cu)
 const char* igks_noalloc_last_error_();
 
+static_assert(PF_E == 3, "KIND_THIRD");
+
 namespace {
 
 struct HostMesh {
@@ -560,7 +562,7 @@ static int build(igks_ctx* ctx) {
       while (q0 < sptr[p + 1] && sslot[q0] == SLOT_GHOST) q0++;   // ghosts that come first: the sum's start
       const int m_ = sptr[p + 1] - q0;
       if (m_ > PF_E) { q.kind = KIND_RARE | KIND_CSR; continue; }
-      q.kind = m_ | (m_ > 2 ? KIND_RARE : 0);
+      q.kind = m_ | (m_ > 2 ? KIND_THIRD : 0);
       for (int e = 0; e < m_; e++) {
         if (sslot[q0 + e] < 0) q.kind |= KIND_RARE;
         if (sslot[q0 + e] >= ring) q.kind |= KIND_SIDE;

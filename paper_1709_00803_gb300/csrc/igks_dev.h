@@ -59,7 +59,8 @@ constexpr int PF_E = 3;              // stencil entries held per sweep record
 // consecutive records start on distinct 32-byte bank groups.
 constexpr int SLOT_GLOBAL = -1, SLOT_GHOST = -2;
 constexpr int KIND_COUNT = 7;        // entries
-constexpr int KIND_RARE = 16;        // more than two entries, a ghost, or a neighbour in global memory
+constexpr int KIND_THIRD = 8;        // a third entry, all three in ring or side slots
+constexpr int KIND_RARE = 16;        // a ghost, or a neighbour in global memory
 constexpr int KIND_SIDE = 32;        // a side slot (used by staged solves only)
 constexpr int KIND_CSR = 64;         // more than PF_E entries: the CSR stencil (KIND_RARE too)
 struct alignas(16) SweepStat { int i, kind, pb, spill; int slot[PF_E], pad; };
@@ -218,7 +219,7 @@ constexpr int N_KERNEL_KINDS = 11;   // kernels of one iteration (the wide sweep
 constexpr int ring_slots(int t) { return t == 4 ? 2048 : 1024; }
 constexpr int SIDE = 32;             // side slots of a level (two sets, by the level's parity)
 constexpr int zero_slot(int t) { return ring_slots(t) + 2 * SIDE; }
-constexpr int NARROW_THREADS = 256;  // cell threads of the narrow sweeps (two per cell of a level)
+constexpr int NARROW_THREADS = 256;  // cell threads of the narrow sweeps at most (two per cell of a level)
 constexpr int DEFAULT_WAIT_LIMIT = 1 << 24;   // spins of a device wait (about a second)
 constexpr int MAX_BATCH_GRAPH_ITERS = 64;     // iterations captured in one whole-batch graph at most
 constexpr int WIDE_MAX_LEVELS = 64;  // automatic choice: wide schedule up to this many levels

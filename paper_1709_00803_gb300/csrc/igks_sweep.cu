@@ -24,6 +24,7 @@
 #include <cooperative_groups.h>
 #include <float.h>
 
+#include <algorithm>
 #include <cstddef>
 #include <type_traits>
 
@@ -503,18 +504,24 @@ __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int
 //  - the cell warps do nothing else: a warp of its own issues the bulk copies that bring the
 //    records into shared memory (cp.async.bulk, chunks of 32 or 64 positions on an mbarrier each),
 //    other warps take the finished increments from the ring to global memory one level
-//    later and fetch the increments that left the ring ahead of their level. A cell's record
-//    is in registers when its level begins.
+//    later, and one fetches the increments that left the ring ahead of their level.
+//  - two sets of cell warps take the levels in turn: while one computes a level, the other
+//    has the next level's records in registers and its ring addresses formed, and waits.
+//    (One set that read its next records before the level barrier: FP32 195 + 209 us below,
+//    double-float 360 + 385.) With six warps a set the registers suffice without spills.
 //  - flux increments go to global memory only for the cells that a later cell reads there.
 //  - the ring holds the 13 values of a cell as 12 + 1: x fluxes, y fluxes and increments of
 //    the four mean-flow components (a lane reads its two of each with one vector load; 12
 //    values are 48 or 96 bytes, which puts consecutive cells on distinct banks), SA apart.
 // Forward + backward on the 20,480-cell hybrid plate (351 levels each way), against one
 // thread per cell that read its record inside the level and stored its results itself:
-// FP32 401 + 418 -> 195 + 209 us, double-float 592 + 719 -> 360 + 385, FP64 1192 + 1417 ->
-// 754 + 742 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
+// FP32 401 + 418 -> 184 + 156 us, double-float 592 + 719 -> 344 + 316, FP64 1192 + 1417 ->
+// 756 + 695 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
 // 60,160-cell O-mesh (605 levels; every level has a seam cell whose neighbour left the ring
-// 300 levels ago) FP32 946 + 895 -> 504 + 580 us.
+// 300 levels ago) FP32 946 + 895 -> 490 + 518 us; 5,003 cells of plate 160 + 188 -> 64 + 61.
+// Thin levels (the plate's) end when the store warps have read the level before: store warps
+// outside the level barrier, polling a counter, were no faster (184 + 170, 65 + 65 us; the
+// polls load the shared memory the cells wait for).
 
 // With a cluster of C blocks per solve (C > 1), position q of the solve belongs to block
 // q % C and its increments sit in that block's ring, read through distributed shared
@@ -570,7 +577,8 @@ __device__ __forceinline__ void bulk_g2s(unsigned dst, const void* src, unsigned
 // cluster, reads its records and what left the ring from global memory. CHUNK: an FP32
 // level takes 0.5 us, so the copies come in fewer, larger pieces.
 constexpr int LVL_SMEM = 2048;
-constexpr int STORE_WARPS = 3;
+template <class T>
+constexpr int STORE_WARPS = sizeof(T) == 4 ? 3 : 2;
 template <class T>
 struct Smem {
   static constexpr int SLOTS = ring_slots((int)sizeof(T)), ZERO = zero_slot((int)sizeof(T)), ALL = ZERO + 1;
@@ -633,13 +641,16 @@ __device__ __forceinline__ void load_rec(LaneRec<T>& o, const SweepRec<T>* dy, i
 template <class T>
 struct LaneNb { T x0, x1, y0, y1, w0, w1, w4; };
 
-template <class T, int C>
-__device__ __forceinline__ void ring_read(LaneNb<T>& o, const T* ring, const T* ring4, int slot, int lane) {
-  const T* b = ring_of<T, C>(ring, slot) + slot * 12 + 2 * lane;
+template <class T>
+__device__ __forceinline__ void ring_read_at(LaneNb<T>& o, const T* b, const T* b4) {
   const Pair<T> x = *reinterpret_cast<const Pair<T>*>(b), y = *reinterpret_cast<const Pair<T>*>(b + 4),
                 w = *reinterpret_cast<const Pair<T>*>(b + 8);
   o.x0 = x.a; o.x1 = x.b; o.y0 = y.a; o.y1 = y.b; o.w0 = w.a; o.w1 = w.b;
-  o.w4 = ring_of<T, C>(ring4, slot)[slot];
+  o.w4 = *b4;
+}
+template <class T, int C>
+__device__ __forceinline__ void ring_read(LaneNb<T>& o, const T* ring, const T* ring4, int slot, int lane) {
+  ring_read_at<T>(o, ring_of<T, C>(ring, slot) + slot * 12 + 2 * lane, ring_of<T, C>(ring4, slot) + slot);
 }
 
 template <class T>
@@ -694,13 +705,12 @@ __device__ __forceinline__ LaneOut<T> lane_finish(const LaneRec<T>& rc, T acc0, 
 }
 
 template <class T>
-__device__ __forceinline__ void ring_put(T* ring, T* ring4, int slot, const LaneOut<T>& o, int lane) {
-  T* b = ring + slot * 12;
+__device__ __forceinline__ void ring_put(T* b, T* b4, const LaneOut<T>& o, int lane) {
   Pair<T>* f = reinterpret_cast<Pair<T>*>(b + 4 * lane);
   f[0] = Pair<T>{o.f[0], o.f[1]};
   f[1] = Pair<T>{o.f[2], o.f[3]};
   *reinterpret_cast<Pair<T>*>(b + 8 + 2 * lane) = Pair<T>{o.w0, o.w1};
-  if (lane) ring4[slot] = o.w4;
+  if (lane) *b4 = o.w4;
 }
 
 // increments to global memory: the forward one into the cell's backward record (at = its
@@ -791,28 +801,56 @@ __device__ __forceinline__ void apply_ghost(const Dev& d, T& a0, T& a1, T& a4, c
   if (sa_on) bwd_sa<T>(a4, ((const T*)d.gprim)[-1 - j], m4);
 }
 
-// The increments of the cell at position p (its record in rc; co: the record's coefficients
-// in memory). rare: the kinds that take the general path (with the side slots' when the solve
-// is not staged). Called by whole warps; a thread without a cell of its own (valid = false) works
-// on a copy of another's and stores nothing.
-template <class T, bool FWD, int C>
+// Where a cell's ring reads and writes go, known before its level begins
+struct RingAt {
+  int nb[2], nb4[2], put, put4;
+};
+template <class T>
+__device__ __forceinline__ RingAt ring_at(const LaneRec<T>& rc, int q, int lane) {
+  RingAt a;
+  const int slot = q & (Smem<T>::SLOTS - 1);
+#pragma unroll
+  for (int e = 0; e < 2; e++) {
+    a.nb4[e] = max(rc.slot[e], 0);
+    a.nb[e] = a.nb4[e] * 12 + 2 * lane;
+    asm volatile("" : "+r"(a.nb[e]), "+r"(a.nb4[e]));   // here, not after the level barrier
+  }
+  a.put4 = slot;
+  a.put = slot * 12;
+  asm volatile("" : "+r"(a.put), "+r"(a.put4));
+  return a;
+}
+
+// The increments of the cell at position p (its record in rc). rare: the kinds that take the
+// general path (with the side slots' when the solve is not staged). co2(): the third entry's
+// coefficients in memory. Called by whole warps; a thread without a cell of its own (valid =
+// false) works on a copy of another's and stores nothing.
+template <class T, bool FWD, int C, class Co2>
 __device__ __forceinline__ LaneOut<T> lane_cell(const Dev& d, T* ring, T* ring4, int rare, const LaneRec<T>& rc,
-                                                const T* co, int p, int slot, int lane, bool valid, bool sa_on) {
+                                                const RingAt& at, int p, int lane, bool valid, bool sa_on, Co2 co2) {
   T acc0 = rc.a0, acc1 = rc.a1, acc4 = rc.a4;
   LaneNb<T> nb[2];
 #pragma unroll
-  for (int e = 0; e < 2; e++) ring_read<T, C>(nb[e], ring, ring4, max(rc.slot[e], 0), lane);
+  for (int e = 0; e < 2; e++)
+    ring_read_at<T>(nb[e], ring_of<T, C>(ring, at.nb4[e]) + at.nb[e], ring_of<T, C>(ring4, at.nb4[e]) + at.nb4[e]);
   if (!(rc.kind & rare)) {
 #pragma unroll
     for (int e = 0; e < 2; e++) apply_entry<T, FWD>(acc0, acc1, acc4, rc.co[e], nb[e], sa_on);
+    if (rc.kind & KIND_THIRD) {
+      alignas(16) T c[4];
+      load_co<T>(c, co2());
+      ring_read<T, C>(nb[0], ring, ring4, rc.slot[2], lane);
+      apply_entry<T, FWD>(acc0, acc1, acc4, c, nb[0], sa_on);
+    }
   } else if (!(rc.kind & KIND_CSR)) {
+    const SweepRec<T>* recs = (const SweepRec<T>*)(FWD ? d.frec : d.brec);
     const int* js = (FWD ? d.fj : d.bj)[p].j;
     const int slots = rare & KIND_SIDE ? Smem<T>::SLOTS : Smem<T>::ALL;
 #pragma unroll 1
     for (int e = 0; e < (rc.kind & KIND_COUNT); e++) {
       const int sl = e == 0 ? rc.slot[0] : e == 1 ? rc.slot[1] : rc.slot[2];
       alignas(16) T c[4];
-      load_co<T>(c, co + 4 * e);
+      load_co<T>(c, recs[p].co[e]);
       if (!FWD && sl == SLOT_GHOST) {
         apply_ghost<T>(d, acc0, acc1, acc4, c, js[e], rc.m4, lane, sa_on);
         continue;
@@ -830,7 +868,7 @@ __device__ __forceinline__ LaneOut<T> lane_cell(const Dev& d, T* ring, T* ring4,
   __syncwarp();
   const LaneOut<T> o = lane_finish<T, FWD>(rc, acc0, acc1, acc4, lane, sa_on);
   if (valid) {
-    ring_put<T>(ring, ring4, slot, o, lane);
+    ring_put<T>(ring + at.put, ring4 + at.put4, o, lane);
     if (rc.spill) store_spill<T, FWD>(d, rc.i, o, lane);
   }
   return o;
@@ -883,9 +921,13 @@ __device__ __forceinline__ void ghost_pass(const Dev& d, int s, int first, int s
   }
 }
 
-// level barrier of the cell and store warps
-__device__ __forceinline__ void bar_levels(int threads) {
-  asm volatile("bar.sync 1, %0;\n" ::"r"(threads) : "memory");
+// Level barriers (named, 1 and 2 by the level's parity): the warps that worked on a level
+// arrive, the others wait.
+__device__ __forceinline__ void bar_wait(int id, int threads) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
 }
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
@@ -898,18 +940,20 @@ __device__ __forceinline__ void st_release(int* p, int v) {
 
 // The sweep of one solve. Positions q are counted from the solve's first; level k is
 // [lv(k), lv(k + 1)). With one block per solve the warps have roles:
-//  - cell warps: two threads per cell of level k; then they read the records of level k + 1
-//    (from shared memory as far as they have landed, the others from global memory);
+//  - cell warps: two threads per cell of a level; SETS sets of them take the levels in turn. A
+//    set reads its next records (from shared memory as far as they have landed, the others
+//    from global memory) before it waits for the level before, so with two sets nothing but
+//    the ring reads, the arithmetic and the ring stores lies between two levels;
 //  - store warps: the increments of level k to global memory during level k + 1 (their ring
-//    slots are not reused before level k + 2: two levels fit the ring); the first of them
-//    also fetches increments that left the ring: it reads them during level k for level
-//    k + 2 and puts them into the side slots during level k + 1;
+//    slots are not reused before level k + 2: two levels fit the ring);
+//  - the side warp fetches increments that left the ring: it reads them during level k for
+//    level k + 2 and puts them into the side slots during level k + 1;
 //  - the copy warp: a chunk's buffer is free once all its positions lie in finished levels;
 //    it issues chunks as buffers become free and counts the records that have landed. It
 //    runs beside the level barriers, and nobody waits for it. A chunk that has not landed
 //    after wait_limit tries marks the solve IGKS_TIMEOUT (the update leaves its state
 //    untouched); the warp then waits for the other copies in flight and ends.
-template <class T, bool FWD, int C>
+template <class T, bool FWD, int C, int SETS>
 __device__ __forceinline__ void sweep_narrow(const Dev& d) {
   using S = Smem<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -934,7 +978,9 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
   const int pbase = glv[0], np = glv[nl] - pbase;
   const SweepRec<T>* grec = (const SweepRec<T>*)(FWD ? d.frec : d.brec) + pbase;
   const int tid = threadIdx.x;
-  const int nct = C == 1 ? (int)blockDim.x - 32 * (STORE_WARPS + 1) : (int)blockDim.x;   // cell threads
+  constexpr int NST = 32 * STORE_WARPS<T>;
+  const int nct = C == 1 ? (int)blockDim.x - NST - 64 : (int)blockDim.x;   // cell threads
+  const int nbar = nct + NST + 32;                                 // threads of a level barrier
   const bool lvs = nl + 3 < LVL_SMEM;                              // level offsets in shared memory
   int wide = 0;
   for (int k = tid; k <= nl + 2; k += blockDim.x) {
@@ -951,87 +997,111 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
   auto lv = [&](int k) { return lvs ? slv[k] : glv[min(k, nl)] - pbase; };
 
   if (tid < nct) {
-    const int lane = tid & 1, w0 = (tid & 31) / 2 * C, own = C * (tid >> 1), step = C * nct / 2;
+    const int set = tid / (nct / SETS), t = tid - set * (nct / SETS);
+    const int lane = t & 1, w0 = (t & 31) / 2 * C, own = C * (t >> 1), step = C * (nct / SETS) / 2;
     const int rare = staged ? KIND_RARE : KIND_RARE | KIND_SIDE;
     LaneRec<T> rc;
     auto fetch = [&](int q, int landed) {
       if (q < landed) load_rec<T, FWD>(rc, srec + q % S::NREC, lane);
       else load_rec<T, FWD>(rc, grec + q, lane);
     };
-    int e = lv(1), en = lv(2), q = first_own<C>(0, r) + own;
-    if (q - w0 < e) fetch(min(q, e - 1), 0);                       // a warp works if its first cell exists
-    for (int k = 0; k < nl; k++) {
-      const int ef = lv(k + 3);
+    for (int k = set; k < nl; k += SETS) {
+      const int b = lv(k), e = lv(k + 1);
+      int q = first_own<C>(b, r) + own;
       const int landed = C == 1 ? ld_acquire(landed_p) : 0;
-      while (q - w0 < e) {               // more than one round in a level wider than the block
+      RingAt at;
+      auto next = [&] {                  // the record of position q and its places in the ring
+        fetch(min(q, e - 1), landed);
+        at = ring_at<T>(rc, q, lane);
+      };
+      const bool act = q - w0 < e;       // a warp works if its first cell exists
+      if (act) next();
+      if (C == 1 && k > 0) bar_wait(2 - (k & 1), nbar);            // level k - 1 is finished
+      bool global = !staged;             // increments stored to global memory that others may read
+      if (act) do {                      // more than one round in a level wider than the set
         const bool valid = q < e;
         const int qc = min(q, e - 1);
-        const T* co = qc < landed ? srec[qc % S::NREC].co[0] : grec[qc].co[0];
-        const LaneOut<T> o = lane_cell<T, FWD, C>(d, ring, ring4, rare, rc, co, pbase + qc, q & (S::SLOTS - 1), lane,
-                                                  valid, sa_on);
+        const LaneOut<T> o = lane_cell<T, FWD, C>(
+            d, ring, ring4, rare, rc, at, pbase + qc, lane, valid, sa_on,
+            [&] { return qc < landed ? srec[qc % S::NREC].co[2] : grec[qc].co[2]; });
         if (C > 1 || !staged) {          // no store warps, or levels that may overrun the ring
           const T p0 = shfl_pair(o.w0), p1 = shfl_pair(o.w1);
           const T w[4] = {o.w0, o.w1, p0, p1};
           if (valid && lane == 0) store_inc<T, FWD>(d, FWD ? rc.pb : rc.i, w, o.w4);
         }
+        global |= rc.spill != 0;
         q += step;
-        if (q - w0 < e) fetch(min(q, e - 1), landed);
-      }
-      q = first_own<C>(e, r) + own;
-      if (q - w0 < en) fetch(min(q, en - 1), landed);
-      if constexpr (C == 1) bar_levels(nct + 32 * STORE_WARPS);
-      else cg::this_cluster().sync();    // release/acquire over the cluster's shared and global writes
-      e = en; en = ef;
+        if (q - w0 >= e) break;
+        next();
+      } while (true);
+      if (C == 1 && global) __threadfence_block();
+      if constexpr (C > 1) cg::this_cluster().sync();   // release/acquire over the cluster's shared and global writes
+      else if (SETS > 1) bar_arrive(1 + (k & 1), nbar);
+      else if (k == nl - 1) bar_wait(1 + (k & 1), nbar);
     }
-  } else if (tid < nct + 32 * STORE_WARPS) {
-    const int t = tid - nct, n = d.nc_pad;
+    if (SETS > 1 && set != (nl - 1) % SETS) bar_wait(1 + ((nl - 1) & 1), nbar);
+  } else if (tid < nct + NST) {
+    const int t = tid - nct;
+    auto at = [&](int q) { return FWD ? grec[q].st.pb : grec[q].st.i; };
+    constexpr int ROUNDS = 3;                                      // positions whose targets are read a level ahead
+    int b = 0, e = 0, en = lv(1), next[ROUNDS];
+#pragma unroll
+    for (int j = 0; j < ROUNDS; j++) next[j] = t + j * NST < en ? at(t + j * NST) : 0;
+    for (int k = 0; k <= nl; k++) {                                // stores level k - 1
+      if (staged) {
+        if (t == 0) st_release(progress, k);                       // levels below k are finished
+        auto put = [&](int q, int x) {
+          const int slot = q & (S::SLOTS - 1);
+          alignas(16) T w[4];
+          load_co<T>(w, ring + slot * 12 + 8);
+          store_inc<T, FWD>(d, x, w, ring4[slot]);
+        };
+#pragma unroll
+        for (int j = 0; j < ROUNDS; j++) {
+          const int x = next[j];
+          if (e + t + j * NST < en) next[j] = at(e + t + j * NST);
+          if (b + t + j * NST < e) put(b + t + j * NST, x);
+        }
+        for (int q = b + t + ROUNDS * NST; q < e; q += NST) put(q, at(q));
+      }
+      if (k == nl) break;
+      bar_wait(1 + (k & 1), nbar);
+      b = e; e = en; en = lv(k + 2);
+    }
+  } else if (tid < nct + NST + 32) {
+    const int t = tid - nct - NST, n = d.nc_pad;
+    static_assert(SIDE == 32, "one side slot a thread");
     const int* sp = (FWD ? d.fside_ptr : d.bside_ptr) + l0;
     const int* sj = FWD ? d.fside_j : d.bside_j;
     const T* dF = (const T*)d.dF;
     const T* dWv = (const T*)(FWD ? d.dWs : d.dW);
-    auto at = [&](int q) { return FWD ? grec[q].st.pb : grec[q].st.i; };
-    int b = 0, e = 0, en = lv(1), next = t < en ? at(t) : 0;
     // side slots, a step a level: offsets (level k + 4), cell (k + 3), increments (k + 2), slot (k + 1)
-    const bool side = t < SIDE && staged;
     int pa = 0, pb = 0, j = -1, jv = -1;
     T v[13];
-    if (side && nl > 3) { pa = sp[3]; pb = sp[4]; }
-    for (int k = 0; k <= nl; k++) {                                // stores level k - 1
+    if (staged && nl > 3) { pa = sp[3]; pb = sp[4]; }
+    for (int k = 0; k < nl; k++) {
       if (staged) {
-        if (t == 0) st_release(progress, k);                       // levels below k are finished
-        const int ix = next;
-        if (e + t < en) next = at(e + t);
-        for (int q = b + t; q < e; q += 32 * STORE_WARPS) {
-          const int x = q == b + t ? ix : at(q), slot = q & (S::SLOTS - 1);
-          alignas(16) T w[4];
-          load_co<T>(w, ring + slot * 12 + 8);
-          store_inc<T, FWD>(d, x, w, ring4[slot]);
-        }
-        if (side) {
-          if (jv >= 0) {
-            const int slot = S::SLOTS + ((k + 1) & 1) * SIDE + t;
+        if (jv >= 0) {
+          const int slot = S::SLOTS + ((k + 1) & 1) * SIDE + t;
 #pragma unroll
-            for (int c = 0; c < 12; c++) ring[slot * 12 + c] = v[c];
-            ring4[slot] = v[12];
-          }
-          jv = j;
-          if (jv >= 0) {
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-              v[c] = dF[2 * c * n + jv];
-              v[4 + c] = dF[(2 * c + 1) * n + jv];
-              v[8 + c] = dWv[c * n + jv];
-            }
-            v[12] = dWv[4 * n + jv];
-          }
-          j = pa + t < pb ? sj[pa + t] : -1;
-          if (k + 5 <= nl) { pa = sp[k + 4]; pb = sp[k + 5]; }
-          else pa = pb;
+          for (int c = 0; c < 12; c++) ring[slot * 12 + c] = v[c];
+          ring4[slot] = v[12];
         }
+        jv = j;
+        if (jv >= 0) {
+#pragma unroll
+          for (int c = 0; c < 4; c++) {
+            v[c] = dF[2 * c * n + jv];
+            v[4 + c] = dF[(2 * c + 1) * n + jv];
+            v[8 + c] = dWv[c * n + jv];
+          }
+          v[12] = dWv[4 * n + jv];
+        }
+        j = pa + t < pb ? sj[pa + t] : -1;
+        if (k + 5 <= nl) { pa = sp[k + 4]; pb = sp[k + 5]; }
+        else pa = pb;
       }
-      if (k == nl) break;
-      bar_levels(nct + 32 * STORE_WARPS);
-      b = e; e = en; en = lv(k + 2);
+      bar_wait(1 + (k & 1), nbar);
     }
   } else if (staged && (tid & 31) == 0) {
     constexpr int CHUNK = S::CHUNK;
@@ -1080,11 +1150,18 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
   }
 }
 
+// Cell threads of one set at most: what lets the registers of both sets fit (FP32 96 a
+// thread, the 8-byte types 128). A level wider than a set takes rounds.
+constexpr int SETS = 2;
+template <class T>
+constexpr int SET_THREADS = sizeof(T) == 4 ? 224 : 192;
+template <class T>
+constexpr int block_threads(int set) { return SETS * set + 32 * STORE_WARPS<T> + 64; }
 template <class T, bool FWD>
-__global__ void __launch_bounds__(NARROW_THREADS + 32 * (STORE_WARPS + 1), 1)
-k_sweep_block(const __grid_constant__ Dev d) { sweep_narrow<T, FWD, 1>(d); }
+__global__ void __launch_bounds__(block_threads<T>(SET_THREADS<T>), 1)
+k_sweep_block(const __grid_constant__ Dev d) { sweep_narrow<T, FWD, 1, SETS>(d); }
 template <class T, bool FWD, int C>
-__global__ void __launch_bounds__(NARROW_THREADS) k_sweep_cluster(const __grid_constant__ Dev d) { sweep_narrow<T, FWD, C>(d); }
+__global__ void __launch_bounds__(NARROW_THREADS) k_sweep_cluster(const __grid_constant__ Dev d) { sweep_narrow<T, FWD, C, 1>(d); }
 
 // ---- wide schedule: one launch per level, all solves ----
 template <class T>
@@ -1158,8 +1235,8 @@ static void launch_narrow(const Dev& d, int threads, cudaStream_t s) {
     case 2: launch_cluster<T, FWD, 2>(d, threads, s); break;
     case 4: launch_cluster<T, FWD, 4>(d, threads, s); break;
     case 8: launch_cluster<T, FWD, 8>(d, threads, s); break;
-    default:   // one block per solve: the cells' threads, the store warps and the copy warp
-      k_sweep_block<T, FWD><<<d.g_nsolve, threads + 32 * (STORE_WARPS + 1), Smem<T>::total, s>>>(d);
+    default:   // one block per solve: the cells' threads, the store, side and copy warps
+      k_sweep_block<T, FWD><<<d.g_nsolve, block_threads<T>(std::min(threads, SET_THREADS<T>)), Smem<T>::total, s>>>(d);
       break;
   }
 }
