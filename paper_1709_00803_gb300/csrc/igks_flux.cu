@@ -222,12 +222,12 @@ __global__ void __launch_bounds__(128, 1) k_flux_moment(Dev d) {
     }
   }
   rot(WcRg, nx, ny, WcR);
-  const double mut_face = 0.5 * (d.mu_t[L] + mtR);
+  const double mut_face = gks_moment::hlf(d.mu_t[L] + mtR);
 
   // ---- Eq. 4-14: the time-integrated flux in the face frame ----
   double Fn[4];
   gks_moment::face_flux(WL, WR, SLn, SLt, SRn, SRt, WcL, WcR, idL, idR, mut_face, dt, fl.c_num, fl.pr_fix,
-                        [&](double h) { return viscosity_h(fl, h); }, Fn);
+                        [&](double h2) { return viscosity_h2(fl, h2); }, Fn);
 
   // ---- back to the global frame, times the face length ----
   d.F[f] = Fn[0] * S;
