@@ -255,6 +255,7 @@ static int setup_groups(igks_ctx* ctx) {
   }
   for (int g = 0; g < G; g++) {
     Dev v = d;
+    v.chained = G == 1 && !ctx->opt.timing;
     const int s0 = cut[g], s1 = cut[g + 1];
     v.g_solve0 = s0; v.g_nsolve = s1 - s0;
     v.g_blk0 = ctx->cell_off[s0] / CELL_BLOCK;

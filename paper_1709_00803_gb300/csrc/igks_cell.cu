@@ -169,6 +169,7 @@ __device__ __forceinline__ void speeds_of(const double* W, double* u, double* v,
 // laminar and eddy viscosity of every cell, and its velocity and sound speed (read by the
 // face spectral radius of both cells of each face)
 __global__ void __launch_bounds__(CELL_BLOCK) k_prep(Dev d) {
+  chain_wait();
   int i = (d.g_blk0 + blockIdx.x) * CELL_BLOCK + threadIdx.x, s;
   if (!cell_live(d, i, &s)) return;
   const DevFlow& fl = d.flow[s];
@@ -220,6 +221,7 @@ __device__ __forceinline__ double face_lambda(const DevFlow& fl, double uL, doub
 // per face: the ghost state of a boundary face (Section II.E) and the face spectral
 // radius lambda_f of Eq. 21 (computed once per face, read by both cells' Lambda sums)
 __global__ void k_ghost(Dev d) {
+  chain_wait();
   int f = d.g_face0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= d.g_face0 + d.g_nface) return;
   int s = d.fsolve[f];
@@ -248,17 +250,18 @@ __global__ void k_ghost(Dev d) {
 }
 
 void launch_prep(const Dev& d, cudaStream_t s) {
-  k_prep<<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
+  launch_chained(d.chained, k_prep, d.g_nblk, CELL_BLOCK, 0, s, d);
 }
 
 void launch_ghost(const Dev& d, cudaStream_t s) {
-  if (d.g_nface) k_ghost<<<(d.g_nface + 127) / 128, 128, 0, s>>>(d);
+  if (d.g_nface) launch_chained(d.chained, k_ghost, (d.g_nface + 127) / 128, 128, 0, s, d);
 }
 
 // Least-squares gradients (Eq. 7) of the conserved variables over the face neighbours
 // (ghosts included), the limiter of Eq. 9-10, the vorticity for SA, Lambda_i from the face
 // spectral radii and the per-solve minimum explicit time step (Eq. 23).
 __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
+  chain_wait();
   const int blk = d.g_blk0 + blockIdx.x;
   int i = blk * CELL_BLOCK + threadIdx.x, s = -1;
   bool live = cell_live(d, i, &s);
@@ -383,13 +386,14 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
 }
 
 void launch_gradient(const Dev& d, cudaStream_t s) {
-  k_gradient<<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
+  launch_chained(d.chained, k_gradient, d.g_nblk, CELL_BLOCK, 0, s, d);
 }
 
 // Residual M_i = -(1/dt) sum over the faces of cell i (ascending face order) of the signed
 // face flux (Eq. 16), the SA right-hand side Omega Sr + R (Eq. 27-28a), the SA diagonal
 // without its time term, and per-block partial norms of M_rho.
 __global__ void __launch_bounds__(CELL_BLOCK) k_residual(Dev d) {
+  chain_wait();
   const int blk = d.g_blk0 + blockIdx.x;
   int i = blk * CELL_BLOCK + threadIdx.x, s = -1;
   bool live = cell_live(d, i, &s);
@@ -474,6 +478,7 @@ void launch_residual(const Dev& d, cudaStream_t s) {
 // partial norms added in a fixed order (thread t takes blocks t, t + NORM_THREADS, ..., then
 // a tree): one thread walking 235 blocks took 36 us.
 __global__ void __launch_bounds__(NORM_THREADS) k_norms(Dev d) {
+  chain_wait();
   const int s = d.g_solve0 + blockIdx.x;
   SolveState& st = d.st[s];
   if (st.state != 0) return;
@@ -506,10 +511,11 @@ __global__ void __launch_bounds__(NORM_THREADS) k_norms(Dev d) {
 }
 
 void launch_norms(const Dev& d, cudaStream_t s) {
-  k_norms<<<d.g_nsolve, NORM_THREADS, 0, s>>>(d);
+  launch_chained(d.chained, k_norms, d.g_nsolve, NORM_THREADS, 0, s, d);
 }
 
 __global__ void k_end_iter(Dev d) {
+  chain_wait();
   int s = d.g_solve0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= d.g_solve0 + d.g_nsolve) return;
   SolveState& st = d.st[s];
@@ -528,7 +534,7 @@ __global__ void k_end_iter(Dev d) {
 }
 
 void launch_end_iter(const Dev& d, cudaStream_t s) {
-  k_end_iter<<<(d.g_nsolve + 63) / 64, 64, 0, s>>>(d);
+  launch_chained(d.chained, k_end_iter, (d.g_nsolve + 63) / 64, 64, 0, s, d);
 }
 
 // ===================================================================================

@@ -191,6 +191,7 @@ struct Dev {
   // cells, per-face kernels faces [g_face0, g_face0 + g_nface), per-solve kernels and the
   // narrow sweeps solves [g_solve0, g_solve0 + g_nsolve).
   int g_blk0, g_nblk, g_face0, g_nface, g_solve0, g_nsolve;
+  int chained;                   // launch_chained: one group, no events between the kernels
 };
 
 // ---- launches (igks_kernels.cu / igks_flux.cu) ----
@@ -213,6 +214,32 @@ void launch_end_iter(const Dev& d, cudaStream_t s);
 // check a staged [5][nc_pad] state per solve (bad[s] = 1: non-physical) and copy the
 // solves that pass into W
 void launch_set_state(const Dev& d, const double* staged, int* bad, cudaStream_t s);
+// Launches of an iteration are chained (programmatic dependent launch): once all blocks of a
+// kernel run, the blocks of the next one in the stream may take free places, and every thread
+// waits for the end of the kernel before (chain_wait, the first thing in a kernel) and so for
+// all before that. It hides part of the launch latency, 0.5 us a kernel: cavity of 10,000 cells
+// 82.4 -> 79.5 us an explicit iteration, 133 -> 128 with multicolour sweeps (two levels), 1,470 polygons
+// 235 -> 219 (ten levels). Not chained: several groups, which fill the GPU by themselves; the
+// narrow sweeps, which have too few blocks to gain; the residual, whose waiting blocks slow
+// the flux's last wave and the sweeps after it (20,480 cells in mixed precision 493 -> 515 us).
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+inline void launch_chained(bool chained, void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s, A... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k, P(a)...);
+}
 constexpr int N_KERNEL_KINDS = 11;   // kernels of one iteration (the wide sweeps launch per level)
 // shared-memory ring of the narrow sweeps (cells) for a sweep type of t bytes: 13 values a
 // cell, 104 KiB either way (a power of two: any cluster size divides it)

@@ -56,6 +56,7 @@ __device__ __forceinline__ void side_of(const Dev& d, const double* gr, int c, d
 }
 
 __global__ void __launch_bounds__(128, 1) k_flux(Dev d) {
+  chain_wait();
   const int f = d.g_face0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= d.g_face0 + d.g_nface) return;
   const int s = d.fsolve[f];
@@ -146,6 +147,7 @@ __global__ void __launch_bounds__(128, 1) k_flux(Dev d) {
 }
 
 __global__ void __launch_bounds__(128, 1) k_flux_moment(Dev d) {
+  chain_wait();
   const int f = d.g_face0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= d.g_face0 + d.g_nface) return;
   const int s = d.fsolve[f];
@@ -301,8 +303,8 @@ void launch_flux(const Dev& d, int precision, cudaStream_t s) {
   // 35,000 faces on)
   const int b = d.flux_block > 0 ? d.flux_block : 32;
   if (!d.g_nface) return;
-  if (precision == 1) k_flux_moment<<<(d.g_nface + b - 1) / b, b, 0, s>>>(d);
-  else k_flux<<<(d.g_nface + b - 1) / b, b, 0, s>>>(d);
+  if (precision == 1) launch_chained(d.chained, k_flux_moment, (d.g_nface + b - 1) / b, b, 0, s, d);
+  else launch_chained(d.chained, k_flux, (d.g_nface + b - 1) / b, b, 0, s, d);
 }
 
 }  // namespace igks

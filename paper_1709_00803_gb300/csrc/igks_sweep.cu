@@ -206,6 +206,7 @@ __device__ __forceinline__ void store_chunks(void* dst, const void* src) {
 // ---- pre-pass: per-cell constants and the signed stencil of every cell ----
 template <class T>
 __global__ void __launch_bounds__(CELL_BLOCK) k_sweep_prep(Dev d) {
+  chain_wait();
   const int i = (d.g_blk0 + blockIdx.x) * CELL_BLOCK + threadIdx.x;
   if (i >= d.nc_pad) return;
   const int s = d.cell_solve[i];
@@ -438,6 +439,7 @@ __device__ __forceinline__ void bwd_cell(const Dev& d, int i, bool sa_on) {
 // chain, and its FP64 square roots and division are spread over the whole GPU.
 template <class T>
 __global__ void __launch_bounds__(CELL_BLOCK) k_update(Dev d) {
+  chain_wait();
   const int blk = d.g_blk0 + blockIdx.x;
   const int i = blk * CELL_BLOCK + threadIdx.x;
   const int s = d.cell_solve[blk * CELL_BLOCK];   // every block lies in one solve
@@ -1166,6 +1168,7 @@ __global__ void __launch_bounds__(NARROW_THREADS) k_sweep_cluster(const __grid_c
 // ---- wide schedule: one launch per level, all solves ----
 template <class T>
 __global__ void k_sweep_fwd_level(Dev d, int b, int e) {
+  chain_wait();
   const int k = b + blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= e) return;
   const int i = d.wfwd_cells[k];
@@ -1176,6 +1179,7 @@ __global__ void k_sweep_fwd_level(Dev d, int b, int e) {
 
 template <class T>
 __global__ void k_sweep_bwd_level(Dev d, int b, int e) {
+  chain_wait();
   const int k = b + blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= e) return;
   const int i = d.wbwd_cells[k];
@@ -1187,9 +1191,9 @@ __global__ void k_sweep_bwd_level(Dev d, int b, int e) {
 constexpr int WIDE_BLOCK = 128;
 
 void launch_update(const Dev& d, int precision, cudaStream_t s) {
-  if (precision == 1) k_update<float><<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
-  else if (precision == 2) k_update<df64><<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
-  else k_update<double><<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
+  if (precision == 1) launch_chained(d.chained, k_update<float>, d.g_nblk, CELL_BLOCK, 0, s, d);
+  else if (precision == 2) launch_chained(d.chained, k_update<df64>, d.g_nblk, CELL_BLOCK, 0, s, d);
+  else launch_chained(d.chained, k_update<double>, d.g_nblk, CELL_BLOCK, 0, s, d);
 }
 
 template <class T, bool FWD>
@@ -1242,9 +1246,9 @@ static void launch_narrow(const Dev& d, int threads, cudaStream_t s) {
 }
 
 void launch_sweep_prep(const Dev& d, int precision, cudaStream_t s) {
-  if (precision == 1) k_sweep_prep<float><<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
-  else if (precision == 2) k_sweep_prep<df64><<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
-  else k_sweep_prep<double><<<d.g_nblk, CELL_BLOCK, 0, s>>>(d);
+  if (precision == 1) launch_chained(d.chained, k_sweep_prep<float>, d.g_nblk, CELL_BLOCK, 0, s, d);
+  else if (precision == 2) launch_chained(d.chained, k_sweep_prep<df64>, d.g_nblk, CELL_BLOCK, 0, s, d);
+  else launch_chained(d.chained, k_sweep_prep<double>, d.g_nblk, CELL_BLOCK, 0, s, d);
 }
 
 void launch_sweep_fwd(const Dev& d, int precision, int threads, cudaStream_t s) {
@@ -1252,9 +1256,9 @@ void launch_sweep_fwd(const Dev& d, int precision, int threads, cudaStream_t s) 
     for (int l = 0; l < d.n_wfwd; l++) {
       const int b = d.h_wfwd_ptr[l], e = d.h_wfwd_ptr[l + 1];
       const int g = (e - b + WIDE_BLOCK - 1) / WIDE_BLOCK;
-      if (precision == 1) k_sweep_fwd_level<float><<<g, WIDE_BLOCK, 0, s>>>(d, b, e);
-      else if (precision == 2) k_sweep_fwd_level<df64><<<g, WIDE_BLOCK, 0, s>>>(d, b, e);
-      else k_sweep_fwd_level<double><<<g, WIDE_BLOCK, 0, s>>>(d, b, e);
+      if (precision == 1) launch_chained(d.chained, k_sweep_fwd_level<float>, g, WIDE_BLOCK, 0, s, d, b, e);
+      else if (precision == 2) launch_chained(d.chained, k_sweep_fwd_level<df64>, g, WIDE_BLOCK, 0, s, d, b, e);
+      else launch_chained(d.chained, k_sweep_fwd_level<double>, g, WIDE_BLOCK, 0, s, d, b, e);
     }
     return;
   }
@@ -1268,9 +1272,9 @@ void launch_sweep_bwd(const Dev& d, int precision, int threads, cudaStream_t s) 
     for (int l = 0; l < d.n_wbwd; l++) {
       const int b = d.h_wbwd_ptr[l], e = d.h_wbwd_ptr[l + 1];
       const int g = (e - b + WIDE_BLOCK - 1) / WIDE_BLOCK;
-      if (precision == 1) k_sweep_bwd_level<float><<<g, WIDE_BLOCK, 0, s>>>(d, b, e);
-      else if (precision == 2) k_sweep_bwd_level<df64><<<g, WIDE_BLOCK, 0, s>>>(d, b, e);
-      else k_sweep_bwd_level<double><<<g, WIDE_BLOCK, 0, s>>>(d, b, e);
+      if (precision == 1) launch_chained(d.chained, k_sweep_bwd_level<float>, g, WIDE_BLOCK, 0, s, d, b, e);
+      else if (precision == 2) launch_chained(d.chained, k_sweep_bwd_level<df64>, g, WIDE_BLOCK, 0, s, d, b, e);
+      else launch_chained(d.chained, k_sweep_bwd_level<double>, g, WIDE_BLOCK, 0, s, d, b, e);
     }
     return;
   }
