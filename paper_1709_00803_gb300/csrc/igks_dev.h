@@ -191,6 +191,7 @@ struct Dev {
   // cells, per-face kernels faces [g_face0, g_face0 + g_nface), per-solve kernels and the
   // narrow sweeps solves [g_solve0, g_solve0 + g_nsolve).
   int g_blk0, g_nblk, g_face0, g_nface, g_solve0, g_nsolve;
+  int sweeps;                    // 0: every solve of the group is explicit, the sweeps are not launched
   int chained;                   // launch_chained: one group, no events between the kernels
 };
 

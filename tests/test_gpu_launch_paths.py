@@ -47,3 +47,28 @@ def test_launch_paths_bitwise(name, precision, scheme):
         for a, b in zip(out, ref):
             assert np.isfinite(b).all()
             assert np.array_equal(a, b), (opt, np.abs(a - b).max())
+
+
+@pytest.mark.parametrize("first", [0, 1])
+def test_scheme_changed_after_build(first):
+    """A context whose solves are all explicit launches no sweeps; changing a scheme between
+    iterations changes the launches with it."""
+    from paper_1709_00803_gb300 import igks
+    m, out = G.cavity(24), []
+    for use_graph in (1, 0):
+        ctx = igks.Context(precision=igks.PREC_MIXED, use_graph=use_graph)
+        sid = ctx.mesh_upload(m)
+        for step, scheme in enumerate((first, 1 - first, first)):
+            fl = F.cavity_flow()
+            fl.scheme = scheme
+            ctx.set_flow(sid, fl)
+            if not step:
+                ctx.init_freestream(sid)
+                ctx.set_fields(sid, F.perturbed_state(m, fl, seed=2, amp=0.02))
+            ctx.iterate(3)
+            info = ctx.mesh_info(sid)               # few levels: one launch per level
+            sweeps = 1 + info["levels_fwd"] + info["levels_bwd"]
+            assert ctx.launches_per_iteration() == 8 + (0 if scheme == 1 and use_graph else sweeps)
+        out.append(ctx.get_fields(sid))
+        ctx.destroy()
+    assert np.array_equal(out[0], out[1])
