@@ -192,16 +192,6 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_prep(Dev d) {
   d.pu[i] = u; d.pv[i] = v; d.pc[i] = sqrt(GAMMA * h);
 }
 
-// state of the cell across face f (ghost on a boundary)
-__device__ __forceinline__ void across_W(const Dev& d, int f, int j, double* Wk) {
-  if (j >= 0) {
-    int n = d.nc_pad;
-    for (int v = 0; v < 5; v++) Wk[v] = d.W[v * n + j];
-  } else {
-    for (int v = 0; v < 5; v++) Wk[v] = d.G[v * d.nf + f];
-  }
-}
-
 // face spectral radius lambda_f = |Vbar.n| + cbar (+ viscous term) from the velocities and
 // sound speeds of the two sides, always in the face's own left/right order so both cells
 // get the same bits
@@ -260,41 +250,54 @@ void launch_ghost(const Dev& d, cudaStream_t s) {
 // Least-squares gradients (Eq. 7) of the conserved variables over the face neighbours
 // (ghosts included), the limiter of Eq. 9-10, the vorticity for SA, Lambda_i from the face
 // spectral radii and the per-solve minimum explicit time step (Eq. 23).
-__global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
+//
+// V threads per cell, each with 4 / V of the variables, whose arithmetic is the same and
+// independent of the others'. A warp alone on its scheduler issues an FP64 instruction per 64
+// cycles, four on an SM one per 19: below GRADIENT_SPLIT cells, where one thread per cell
+// leaves an SM one or two warps, four threads per cell are faster (5,040 cells with the smooth
+// limiter 30.7 -> 22.7 us, 1,470 polygons without 16.5 -> 14.4); above it the SMs are busy and
+// the offsets that all four form cost more than the split saves.
+constexpr int GRADIENT_SPLIT = 8192;
+template <int V>
+__global__ void __launch_bounds__(CELL_BLOCK * V) k_gradient(Dev d) {
   chain_wait();
+  constexpr int NV = 4 / V;
   const int blk = d.g_blk0 + blockIdx.x;
-  int i = blk * CELL_BLOCK + threadIdx.x, s = -1;
+  const int v0 = V == 1 ? 0 : threadIdx.x % V;       // the thread's variables: v0 ... v0 + NV - 1
+  int i = blk * CELL_BLOCK + threadIdx.x / V, s = -1;
   bool live = cell_live(d, i, &s);
   unsigned long long dtc = ~0ull;   // bits of the cell's time step
   if (live) {
     const DevFlow& fl = d.flow[s];
     const int n = d.nc_pad;
-    double Wi[5];
-    for (int v = 0; v < 5; v++) Wi[v] = d.W[v * n + i];
+    double Wi[NV];
+#pragma unroll
+    for (int v = 0; v < NV; v++) Wi[v] = d.W[(v0 + v) * n + i];
     double xi = d.cx[i], yi = d.cy[i];
     const bool lim = fl.limiter != 0;
-    double r0[4] = {0, 0, 0, 0}, r1[4] = {0, 0, 0, 0};
-    long long kmax[4], kmin[4];       // extremes over the cell and its neighbours (ord_of)
+    double r0[NV], r1[NV];
+    long long kmax[NV], kmin[NV];       // extremes over the cell and its neighbours (ord_of)
 #pragma unroll
-    for (int v = 0; v < 4; v++) kmax[v] = kmin[v] = ord_of(Wi[v]);
+    for (int v = 0; v < NV; v++) { r0[v] = r1[v] = 0.0; kmax[v] = kmin[v] = ord_of(Wi[v]); }
     double Lam = 0.0;
     for (int k = d.cf_ptr[i]; k < d.cf_ptr[i + 1]; k++) {
       int f = d.cf_face[k];
       int L = d.fL[f], R = d.fR[f];
       int j = (L == i) ? R : L;
-      double Wk[5], xk, yk;
-      across_W(d, f, j, Wk);
+      double Wk[NV], xk, yk;
+#pragma unroll
+      for (int v = 0; v < NV; v++) Wk[v] = j >= 0 ? d.W[(v0 + v) * n + j] : d.G[(v0 + v) * d.nf + f];
       if (j >= 0) { xk = d.cx[j]; yk = d.cy[j]; } else { xk = d.fcx[f]; yk = d.fcy[f]; }
       double dx = xk - xi, dy = yk - yi;
 #pragma unroll
-      for (int v = 0; v < 4; v++) {
+      for (int v = 0; v < NV; v++) {
         double dw = Wk[v] - Wi[v];
         r0[v] += dx * dw;
         r1[v] += dy * dw;
       }
       if (lim)
 #pragma unroll
-        for (int v = 0; v < 4; v++) {
+        for (int v = 0; v < NV; v++) {
           const long long k_ = ord_of(Wk[v]);
           kmax[v] = max(kmax[v], k_);
           kmin[v] = min(kmin[v], k_);
@@ -305,15 +308,17 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
     // the geometry's normal matrix and 1/det (k_lsq_matrix)
     const double A00 = d.lsq[i], A01 = d.lsq[n + i], A11 = d.lsq[2 * n + i], idet = d.lsq[3 * n + i];
     double area = d.area[i];
-    double b[8];
+    double b[2 * NV];
 #pragma unroll
-    for (int v = 0; v < 4; v++) {
+    for (int v = 0; v < NV; v++) {
       b[2 * v] = (A11 * r0[v] - A01 * r1[v]) * idet;
       b[2 * v + 1] = (A00 * r1[v] - A01 * r0[v]) * idet;
-      d.grad[(2 * v) * n + i] = b[2 * v];
-      d.grad[(2 * v + 1) * n + i] = b[2 * v + 1];
+      d.grad[(2 * (v0 + v)) * n + i] = b[2 * v];
+      d.grad[(2 * (v0 + v) + 1) * n + i] = b[2 * v + 1];
     }
-    double phi[4] = {1.0, 1.0, 1.0, 1.0};
+    double phi[NV];
+#pragma unroll
+    for (int v = 0; v < NV; v++) phi[v] = 1.0;
     if (fl.limiter == 1) {
       // Barth-Jespersen: the smallest ratio over the vertices comes from the largest
       // excursion of each sign (correctly rounded division is monotone in the divisor),
@@ -321,12 +326,12 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
       // correctly rounded x / y with 0 < x < y stays below 1, so min(1, x / y) is 1
       // exactly when x >= y and the division is needed only where the limiter acts.
       // Magnitudes of one sign are compared by their bits.
-      unsigned long long up[4] = {0, 0, 0, 0}, dn[4] = {0, 0, 0, 0};
+      unsigned long long up[NV] = {}, dn[NV] = {};
       for (int k = d.cn_ptr[i]; k < d.cn_ptr[i + 1]; k++) {
         int nd = d.cn_node[k];
         double ox = d.xy[nd] - xi, oy = d.xy[d.nn + nd] - yi;
 #pragma unroll
-        for (int v = 0; v < 4; v++) {
+        for (int v = 0; v < NV; v++) {
           const unsigned long long q = bits_of(b[2 * v] * ox + b[2 * v + 1] * oy);
           const unsigned long long m = q & 0x7fffffffffffffffull;
           if (q == m) up[v] = max(up[v], m);
@@ -334,7 +339,7 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
         }
       }
 #pragma unroll
-      for (int v = 0; v < 4; v++) {
+      for (int v = 0; v < NV; v++) {
         const double hi = of_ord(kmax[v]) - Wi[v], lo = Wi[v] - of_ord(kmin[v]);
         if (bits_of(hi) < up[v]) phi[v] = hi / of_bits(up[v]);
         if (bits_of(lo) < dn[v]) {
@@ -345,14 +350,14 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
     } else if (fl.limiter == 2) {
       double h = sqrt(area);
       double eps2 = (fl.venkat_k * h) * (fl.venkat_k * h) * (fl.venkat_k * h);
-      double hi[4], lo[4];
+      double hi[NV], lo[NV];
 #pragma unroll
-      for (int v = 0; v < 4; v++) { hi[v] = of_ord(kmax[v]) - Wi[v]; lo[v] = of_ord(kmin[v]) - Wi[v]; }
+      for (int v = 0; v < NV; v++) { hi[v] = of_ord(kmax[v]) - Wi[v]; lo[v] = of_ord(kmin[v]) - Wi[v]; }
       for (int k = d.cn_ptr[i]; k < d.cn_ptr[i + 1]; k++) {
         int nd = d.cn_node[k];
         double ox = d.xy[nd] - xi, oy = d.xy[d.nn + nd] - yi;
 #pragma unroll
-        for (int v = 0; v < 4; v++) {
+        for (int v = 0; v < NV; v++) {
           double dv = b[2 * v] * ox + b[2 * v + 1] * oy;
           if (bits_of(dv) << 1) {   // not zero
             const double dp = __double2hiint(dv) < 0 ? lo[v] : hi[v];
@@ -364,20 +369,32 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
       }
     }
 #pragma unroll
-    for (int v = 0; v < 4; v++) d.phi[v * n + i] = phi[v];
+    for (int v = 0; v < NV; v++) d.phi[(v0 + v) * n + i] = phi[v];
     if (fl.limiter)   // limited once per cell for the three or four faces that read it
 #pragma unroll
-      for (int v = 0; v < 4; v++) {
-        d.lgrad[(2 * v) * n + i] = phi[v] * b[2 * v];
-        d.lgrad[(2 * v + 1) * n + i] = phi[v] * b[2 * v + 1];
+      for (int v = 0; v < NV; v++) {
+        d.lgrad[(2 * (v0 + v)) * n + i] = phi[v] * b[2 * v];
+        d.lgrad[(2 * (v0 + v) + 1) * n + i] = phi[v] * b[2 * v + 1];
       }
-    const double ir = __drcp_rn(Wi[0]);
-    double u = Wi[1] * ir, vv = Wi[2] * ir;
-    double dudy = (b[3] - u * b[1]) * ir;
-    double dvdx = (b[4] - vv * b[0]) * ir;
-    d.omega[i] = fabs(dvdx - dudy);
-    d.Lam[i] = Lam;
-    dtc = bits_of(fl.cfl_exp * area / Lam);   // positive doubles order like their bits
+    // the cell's first thread: gradients of density and momentum from its neighbour lanes
+    double rx = b[0], ry = b[1], mx, my, mxy, myx;
+    if constexpr (V == 1) {
+      mx = Wi[1]; mxy = b[3];
+      my = Wi[2]; myx = b[4];
+    } else {
+      const unsigned quad = 0xfu << (threadIdx.x & 28);
+      mx = __shfl_sync(quad, Wi[0], 1, 4); mxy = __shfl_sync(quad, b[1], 1, 4);
+      my = __shfl_sync(quad, Wi[0], 2, 4); myx = __shfl_sync(quad, b[0], 2, 4);
+    }
+    if (v0 == 0) {
+      const double ir = __drcp_rn(Wi[0]);
+      double u = mx * ir, vv = my * ir;
+      double dudy = (mxy - u * ry) * ir;
+      double dvdx = (myx - vv * rx) * ir;
+      d.omega[i] = fabs(dvdx - dudy);
+      d.Lam[i] = Lam;
+      dtc = bits_of(fl.cfl_exp * area / Lam);   // positive doubles order like their bits
+    }
   }
   // warp minimum -> at most one atomic per warp; every block lies inside one solve
   dtc = warp_min(dtc);
@@ -386,7 +403,10 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_gradient(Dev d) {
 }
 
 void launch_gradient(const Dev& d, cudaStream_t s) {
-  launch_chained(d.chained, k_gradient, d.g_nblk, CELL_BLOCK, 0, s, d);
+  if (d.g_nblk * CELL_BLOCK <= GRADIENT_SPLIT)
+    launch_chained(d.chained, k_gradient<4>, d.g_nblk, 4 * CELL_BLOCK, 0, s, d);
+  else
+    launch_chained(d.chained, k_gradient<1>, d.g_nblk, CELL_BLOCK, 0, s, d);
 }
 
 // Residual M_i = -(1/dt) sum over the faces of cell i (ascending face order) of the signed
