@@ -517,13 +517,15 @@ __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int
 //    values are 48 or 96 bytes, which puts consecutive cells on distinct banks), SA apart.
 // Forward + backward on the 20,480-cell hybrid plate (351 levels each way), against one
 // thread per cell that read its record inside the level and stored its results itself:
-// FP32 401 + 418 -> 184 + 156 us, double-float 592 + 719 -> 344 + 316, FP64 1192 + 1417 ->
+// FP32 401 + 418 -> 176 + 156 us, double-float 592 + 719 -> 344 + 316, FP64 1192 + 1417 ->
 // 756 + 695 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
 // 60,160-cell O-mesh (605 levels; every level has a seam cell whose neighbour left the ring
-// 300 levels ago) FP32 946 + 895 -> 490 + 518 us; 5,003 cells of plate 160 + 188 -> 64 + 61.
-// Thin levels (the plate's) end when the store warps have read the level before: store warps
-// outside the level barrier, polling a counter, were no faster (184 + 170, 65 + 65 us; the
-// polls load the shared memory the cells wait for).
+// 300 levels ago) FP32 946 + 895 -> 457 + 516 us; 5,003 cells of plate 160 + 188 -> 64 + 60.
+// A level ends when the store warps have stored the level before: one 16-byte store instead of
+// two of 8, and targets of two rounds read ahead instead of three, took FP32 forward from 184
+// and 492 to 176 and 457 us. Store warps that take two levels at a time, in the barrier of every other
+// level, gained 2 us and lost 15; outside the level barrier, polling a counter, they were no
+// faster (184 + 170, 65 + 65 us; the polls load the shared memory the cells wait for).
 
 // With a cluster of C blocks per solve (C > 1), position q of the solve belongs to block
 // q % C and its increments sit in that block's ring, read through distributed shared
@@ -721,8 +723,13 @@ template <class T, bool FWD>
 __device__ __forceinline__ void store_inc(const Dev& d, int at, const T* w, T w4) {
   if constexpr (FWD) {
     T* m = ((SweepRec<T>*)d.brec + at)->m;
-    reinterpret_cast<Pair<T>*>(m)[0] = Pair<T>{w[0], w[1]};
-    reinterpret_cast<Pair<T>*>(m)[1] = Pair<T>{w[2], w[3]};
+    if constexpr (sizeof(T) == 4) {   // one store (double-float and FP64 were 1% slower with two wide ones)
+      alignas(16) const T v[4] = {w[0], w[1], w[2], w[3]};
+      store_chunks<sizeof(v)>(m, v);
+    } else {
+      reinterpret_cast<Pair<T>*>(m)[0] = Pair<T>{w[0], w[1]};
+      reinterpret_cast<Pair<T>*>(m)[1] = Pair<T>{w[2], w[3]};
+    }
     m[4] = w4;
   } else {
     const int n = d.nc_pad;
@@ -1045,7 +1052,7 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
   } else if (tid < nct + NST) {
     const int t = tid - nct;
     auto at = [&](int q) { return FWD ? grec[q].st.pb : grec[q].st.i; };
-    constexpr int ROUNDS = 3;                                      // positions whose targets are read a level ahead
+    constexpr int ROUNDS = sizeof(T) == 4 ? 2 : 3;                 // positions whose targets are read a level ahead
     int b = 0, e = 0, en = lv(1), next[ROUNDS];
 #pragma unroll
     for (int j = 0; j < ROUNDS; j++) next[j] = t + j * NST < en ? at(t + j * NST) : 0;
