@@ -613,6 +613,7 @@ static int build(igks_ctx* ctx) {
   AL(omega, double, nc); AL(mu_l, double, nc); AL(mu_t, double, nc); AL(Lam, double, nc);
   AL(pu, double, nc); AL(pv, double, nc); AL(pc, double, nc); AL(lsq, double, 4 * (size_t)nc);
   AL(M, double, 5 * (size_t)nc); AL(nul, double, nc); AL(sa_diag, double, nc);
+  static_assert(INC_STRIDE * sizeof(float) <= 5 * sizeof(double), "increments of FP32 sweeps");
   AL(dWs, double, 5 * (size_t)nc); AL(dW, double, 5 * (size_t)nc); AL(dF, double, 8 * (size_t)nc);
   AL(fS, double, nf); AL(fnx, double, nf); AL(fny, double, nf); AL(fmx, double, nf); AL(fmy, double, nf);
   AL(fcx, double, nf); AL(fcy, double, nf); AL(fidL, double, nf); AL(fidR, double, nf); AL(fdn, double, nf);
@@ -1102,9 +1103,10 @@ int igks_get_array(igks_ctx* ctx, int32_t solve, int32_t which, double* out) {
       const void* src = which == IGKS_ARR_DWSTAR ? d.dWs : d.dW;
       if (ctx->opt.precision == IGKS_PREC_MIXED) {
         std::vector<float> tmp(5 * (size_t)n);
-        CK(d2h_2d(ctx, tmp.data(), sizeof(float) * n, (const float*)src + ctx->cell_off[solve],
-                  sizeof(float) * ctx->nc_pad, sizeof(float) * n, 5));
-        for (size_t k = 0; k < tmp.size(); k++) out[k] = tmp[k];
+        CK(d2h_2d(ctx, tmp.data(), 5 * sizeof(float), (const float*)src + INC_STRIDE * (size_t)ctx->cell_off[solve],
+                  INC_STRIDE * sizeof(float), 5 * sizeof(float), n));
+        for (int v = 0; v < 5; v++)
+          for (int i = 0; i < n; i++) out[(size_t)v * n + i] = tmp[5 * (size_t)i + v];
         return 0;
       }
       if (ctx->opt.precision == IGKS_PREC_DF64) {   // pairs (hi, lo) of floats
@@ -1370,7 +1372,7 @@ int igks_footprint_bytes(int32_t n_nodes, int32_t n_cells, int32_t n_faces, int3
   const int64_t ncp = (int64_t)(n_cells + CELL_ALIGN - 1) / CELL_ALIGN * CELL_ALIGN;
   // (plus 16 KiB of residual history per solve, in the fixed part below)
   // per padded cell: 62 doubles (state, gradients, speeds, increments, cell constants),
-  // the sweep records (2 x 48 B static, 2 x 272 B per iteration), 9 ints (CSR pointers,
+  // the sweep records (2 x 288 B; the FP32 ones take 2 x 160) and their neighbours' cells, 9 ints (CSR pointers,
   // orders, levels, positions) and 16 B to spare; per CSR entry 60 B (face and node lists, sweep
   // stencil coefficients, maps) + 40 B (one sweep entry); per face 34 doubles + 8 ints; per
   // node 2 doubles; a few hundred bytes per solve

@@ -57,6 +57,7 @@ constexpr int PF_E = 3;              // stencil entries held per sweep record
 // one) are whole 32-byte sectors, so the pre-pass leaves few sectors partly written (with
 // 176-byte records it took 377 us on a batch of 623,000 cells, with these 135 us), and four
 // consecutive records start on distinct 32-byte bank groups.
+constexpr int INC_STRIDE = 8;        // floats of a cell in the FP32 increment arrays (five used)
 constexpr int SLOT_GLOBAL = -1, SLOT_GHOST = -2;
 constexpr int KIND_COUNT = 7;        // entries
 constexpr int KIND_THIRD = 8;        // a third entry, all three in ring or side slots
@@ -114,8 +115,8 @@ struct Dev {
   double* lgrad;            // [8][nc_pad] limited gradients of solves with a limiter, from k_gradient
                             // to k_flux (the memory of sw_st, which the pre-pass writes later)
   double* sa_diag;          // [nc_pad] SA diagonal without the Omega/dt_imp term
-  void* dWs;                // [5][nc_pad] of T (sweep type)
-  void* dW;                 // [5][nc_pad] of T
+  void* dWs;                // increments, T = sweep type: FP32 [nc_pad][INC_STRIDE], else [5][nc_pad]
+  void* dW;                 // the same
   void* dF;                 // [8][nc_pad] of T: increments of the x and y Euler fluxes
   // faces
   const int* fL; const int* fR; const int* fbc; const int* fsolve;

@@ -203,6 +203,35 @@ __device__ __forceinline__ void store_chunks(void* dst, const void* src) {
     reinterpret_cast<uint4*>(dst)[k] = reinterpret_cast<const uint4*>(src)[k];
 }
 
+// A cell's increments in dWs and dW: in FP32 together (INC_STRIDE floats a cell, one 16-byte and
+// one 4-byte access; five rows cost the narrow sweeps' store warps five stores each: the 60,160-cell
+// O-mesh backward 516 -> 453 us), the 8-byte types in rows [5][nc_pad].
+template <class T>
+__device__ __forceinline__ int inc_at(int n, int v, int i) {
+  return sizeof(T) == 4 ? INC_STRIDE * i + v : v * n + i;
+}
+template <class T>
+__device__ __forceinline__ void load_incs(T* w, const T* a, int n, int i) {
+  if constexpr (sizeof(T) == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(a + inc_at<T>(n, 0, i));
+    w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
+    w[4] = a[inc_at<T>(n, 4, i)];
+  } else {
+#pragma unroll
+    for (int v = 0; v < 5; v++) w[v] = a[inc_at<T>(n, v, i)];
+  }
+}
+template <class T>
+__device__ __forceinline__ void store_incs(T* a, int n, int i, const T* w, T w4) {
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(a + inc_at<T>(n, 0, i)) = make_float4(w[0], w[1], w[2], w[3]);
+  } else {
+#pragma unroll
+    for (int v = 0; v < 4; v++) a[inc_at<T>(n, v, i)] = w[v];
+  }
+  a[inc_at<T>(n, 4, i)] = w4;
+}
+
 // ---- pre-pass: per-cell constants and the signed stencil of every cell ----
 template <class T>
 __global__ void __launch_bounds__(CELL_BLOCK) k_sweep_prep(Dev d) {
@@ -298,6 +327,7 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_sweep_prep(Dev d) {
 // the cell's own). On 1470 polygons (10 levels, double-float) the forward sweep takes 66 us,
 // and took 133 us with one entry after the other.
 constexpr int WIDE_E = 4;
+
 template <class T>
 struct WideBatch {
   int j[WIDE_E];
@@ -321,8 +351,7 @@ __device__ __forceinline__ void wide_load(WideBatch<T>& b, const Dev& d, const T
     const int j = use(b.j[e]) ? b.j[e] : i;
 #pragma unroll
     for (int q = 0; q < 8; q++) b.f[e][q] = dF[q * n + j];
-#pragma unroll
-    for (int v = 0; v < 5; v++) b.w[e][v] = dWv[v * n + j];
+    load_incs<T>(b.w[e], dWv, n, j);
   }
 }
 
@@ -335,8 +364,7 @@ __device__ __forceinline__ void wide_finish(const Dev& d, int i, const T* dw, T*
   T o[8];
   delta_flux<T>((T)d.W[i], (T)d.W[n + i], (T)d.W[2 * n + i], c[2 * n + i], c[3 * n + i], c[4 * n + i],
                 dw[0], dw[1], dw[2], dw[3], o);
-#pragma unroll
-  for (int v = 0; v < 5; v++) dWv[v * n + i] = dw[v];
+  store_incs<T>(dWv, n, i, dw, dw[4]);
 #pragma unroll
   for (int q = 0; q < 8; q++) dF[q * n + i] = o[q];
 }
@@ -403,8 +431,7 @@ __device__ __forceinline__ void bwd_cell(const Dev& d, int i, bool sa_on) {
   const T* dF = (const T*)d.dF;
   const T* c = (const T*)d.sw_cell;
   T ws[5];
-#pragma unroll
-  for (int v = 0; v < 5; v++) ws[v] = dWs[v * n + i];
+  load_incs<T>(ws, dWs, n, i);
   T acc[5] = {0, 0, 0, 0, 0};
   const int end = d.cf_ptr[i + 1];
   for (int k0 = d.cf_ptr[i]; k0 < end; k0 += WIDE_E) {
@@ -459,14 +486,16 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_update(Dev d) {
     // explicit scheme (Eq. 15 as Eq. 16): dW = dt M / Omega, in FP64
     const double xf = expl ? __longlong_as_double((long long)d.dt_bits[si]) / d.area[i] : 0.0;
     double num = 0.0, den = 0.0;
+    T dw[5] = {};
+    if (!expl) load_incs<T>(dw, dWo, n, i);
 #pragma unroll
     for (int v = 0; v < 4; v++) {
-      const double dv = expl ? xf * d.M[v * n + i] : to_double(dWo[v * n + i]);
+      const double dv = expl ? xf * d.M[v * n + i] : to_double(dw[v]);
       num += dv * dv;
       den += Wi[v] * Wi[v];
       Wi[v] += dv;
     }
-    Wi[4] += expl ? (d.flow[si].sa_on ? xf * d.M[4 * n + i] : 0.0) : to_double(dWo[4 * n + i]);
+    Wi[4] += expl ? (d.flow[si].sa_on ? xf * d.M[4 * n + i] : 0.0) : to_double(dw[4]);
     if (Wi[4] < 0.0) Wi[4] = 0.0;
     eq40 = num * __drcp_rn(den);
     const double p = Wi[3] - 0.5 * (Wi[1] * Wi[1] + Wi[2] * Wi[2]) * __drcp_rn(Wi[0]);   // for its sign
@@ -517,13 +546,14 @@ __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int
 //    values are 48 or 96 bytes, which puts consecutive cells on distinct banks), SA apart.
 // Forward + backward on the 20,480-cell hybrid plate (351 levels each way), against one
 // thread per cell that read its record inside the level and stored its results itself:
-// FP32 401 + 418 -> 176 + 156 us, double-float 592 + 719 -> 344 + 316, FP64 1192 + 1417 ->
+// FP32 401 + 418 -> 174 + 151 us, double-float 592 + 719 -> 344 + 316, FP64 1192 + 1417 ->
 // 756 + 695 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
 // 60,160-cell O-mesh (605 levels; every level has a seam cell whose neighbour left the ring
-// 300 levels ago) FP32 946 + 895 -> 457 + 516 us; 5,003 cells of plate 160 + 188 -> 64 + 60.
+// 300 levels ago) FP32 946 + 895 -> 455 + 450 us; 5,003 cells of plate 160 + 188 -> 64 + 59.
 // A level ends when the store warps have stored the level before: one 16-byte store instead of
 // two of 8, and targets of two rounds read ahead instead of three, took FP32 forward from 184
-// and 492 to 176 and 457 us. Store warps that take two levels at a time, in the barrier of every other
+// and 492 to 176 and 457 us; a cell's increments side by side in dW (INC_STRIDE) took backward
+// from 155 and 516 to 151 and 450. Store warps that take two levels at a time, in the barrier of every other
 // level, gained 2 us and lost 15; outside the level barrier, polling a counter, they were no
 // faster (184 + 170, 65 + 65 us; the polls load the shared memory the cells wait for).
 
@@ -663,7 +693,7 @@ __device__ __forceinline__ void global_read(LaneNb<T>& o, const Dev& d, const T*
   const T* dF = (const T*)d.dF;
   o.x0 = dF[(4 * lane) * n + j]; o.y0 = dF[(4 * lane + 1) * n + j];
   o.x1 = dF[(4 * lane + 2) * n + j]; o.y1 = dF[(4 * lane + 3) * n + j];
-  o.w0 = dWv[(2 * lane) * n + j]; o.w1 = dWv[(2 * lane + 1) * n + j]; o.w4 = dWv[4 * n + j];
+  o.w0 = dWv[inc_at<T>(n, 2 * lane, j)]; o.w1 = dWv[inc_at<T>(n, 2 * lane + 1, j)]; o.w4 = dWv[inc_at<T>(n, 4, j)];
 }
 
 // a lane's results for one cell: its increments (w4: the SA row, both lanes) and the four
@@ -732,11 +762,7 @@ __device__ __forceinline__ void store_inc(const Dev& d, int at, const T* w, T w4
     }
     m[4] = w4;
   } else {
-    const int n = d.nc_pad;
-    T* dWo = (T*)d.dW;
-#pragma unroll
-    for (int v = 0; v < 4; v++) dWo[v * n + at] = w[v];
-    dWo[4 * n + at] = w4;
+    store_incs<T>((T*)d.dW, d.nc_pad, at, w, w4);
   }
 }
 
@@ -746,9 +772,9 @@ __device__ __noinline__ void store_spill(const Dev& d, int i, LaneOut<T> o, int 
   const int n = d.nc_pad;
   T* dWv = (T*)(FWD ? d.dWs : d.dW);
   T* dF = (T*)d.dF;
-  dWv[(2 * lane) * n + i] = o.w0;
-  dWv[(2 * lane + 1) * n + i] = o.w1;
-  if (lane) dWv[4 * n + i] = o.w4;
+  dWv[inc_at<T>(n, 2 * lane, i)] = o.w0;
+  dWv[inc_at<T>(n, 2 * lane + 1, i)] = o.w1;
+  if (lane) dWv[inc_at<T>(n, 4, i)] = o.w4;
   for (int v = 0; v < 4; v++) dF[(2 * v + lane) * n + i] = o.f[v];
 }
 
@@ -1102,9 +1128,9 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
           for (int c = 0; c < 4; c++) {
             v[c] = dF[2 * c * n + jv];
             v[4 + c] = dF[(2 * c + 1) * n + jv];
-            v[8 + c] = dWv[c * n + jv];
+            v[8 + c] = dWv[inc_at<T>(n, c, jv)];
           }
-          v[12] = dWv[4 * n + jv];
+          v[12] = dWv[inc_at<T>(n, 4, jv)];
         }
         j = pa + t < pb ? sj[pa + t] : -1;
         if (k + 5 <= nl) { pa = sp[k + 4]; pb = sp[k + 5]; }
