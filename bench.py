@@ -55,37 +55,40 @@ FP64_FLOP_PER_SM_CLK = 4.0
 # Algorithmic FP64 work of the gas-kinetic flux per face: 2 kflop, the upper end of the
 # method's own count (two erfc/exp pairs, ten 4x4 moment solves, the moment tables to
 # order 6-7 and the flux assembly); what the kernel executes on top (the instructions
-# inside the library's erfc/exp/divide) does not count as work done
+# inside the library's erfc/exp/divide) does not count as work done; FP64 and double-float
+# solves execute about half of it (igks_gks.cuh), so their rate can pass the peak
 FLUX_ALG_FLOPS_PER_FACE = 2000.0
 # ncu figures per face / per cell of one launch, by workload, with the capture they come
 # from (executed FP64 flops = 2 x DFMA + DADD + DMUL thread instructions; DRAM = read +
-# write bytes). None: not captured for that workload.
+# write bytes); by bytes of the sweep type where precisions differ. None: not captured for
+# that workload.
 NCU = {
-    "naca_batch": {"source": "ncu, k_flux on the first 8 airfoils of the batch (573454 faces), per face",
-                   "flux_exec_flops_per_face": 2230.7, "flux_dram_bytes_per_face": 220.6},
-    "turbulent_plate": {"source": "ncu, k_flux and the one-block-per-solve sweeps on the turbulent flat plate "
+    "naca_batch": {"source": "ncu, k_flux_moment on the first 8 airfoils of the batch (573454 faces), per face",
+                   "flux_exec_flops_per_face": {4: 2125.4}, "flux_dram_bytes_per_face": {4: 198.3}},
+    "turbulent_plate": {"source": "ncu, the flux and the one-block-per-solve sweeps on the turbulent flat plate "
                                   "(35056 faces, 20480 cells)",
-                        "flux_exec_flops_per_face": 2231.0, "flux_dram_bytes_per_face": 186.9,
-                        "sweep_dram_bytes_per_cell": {("k_sweep_fwd", 8): 326.2, ("k_sweep_bwd", 8): 326.7,
-                                                      ("k_sweep_fwd", 4): 194.3, ("k_sweep_bwd", 4): 197.7}},
+                        "flux_exec_flops_per_face": {4: 2121.2, 8: 1058.5},
+                        "flux_dram_bytes_per_face": {4: 168.1, 8: 176.5},
+                        "sweep_dram_bytes_per_cell": {("k_sweep_fwd", 8): 301.5, ("k_sweep_bwd", 8): 300.4,
+                                                      ("k_sweep_fwd", 4): 168.2, ("k_sweep_bwd", 4): 163.9}},
 }
 
 
 def alg_bytes(kernel, t, nc, nf):
     """Algorithmic (compulsory) bytes of one launch: every array the kernel needs streamed
     once, neighbour re-reads from cache. t = bytes of the sweep type."""
-    cell_flux_inputs = 21 * 8          # W 5, gradient 8, limiter 4, centroid 2, mu 2
+    cell_flux_inputs = 17 * 8          # W 5, (limited) gradient 8, centroid 2, mu 2
     per = {
         "k_ghost": nc * (5 * 8 + 2 * 8) + nf * (3 * 4 + 3 * 8 + 8),   # states, viscosities, face ids/geometry, lambda_f
         "k_gradient": nc * (5 * 8 + 2 * 8 + 8 + 8 * 8 + 4 * 8 + 8 + 8) + nf * (2 * 4 + 8 + 8),
         "k_flux": nf * (4 * 4 + 8 * 8 + 10 * 8) + nc * cell_flux_inputs,
         "k_residual": nc * (8 + 8 * 8 + 5 * 8 + 3 * 8) + nf * (6 * 8 + 4 * 8),
-        # records in (48 B static; 13 + 16 T forward, 15 + 16 T backward), increments out
-        "k_sweep_fwd": nc * (48 + 29 * t + 18 * t),
-        "k_sweep_bwd": nc * (48 + 31 * t + 13 * t),
-        # W, M, Lambda, velocity, SA diagonal in; record heads (13 + 15 T) and about four
+        # record in (32 B static, 13 values, three stencil entries of 4), increments out
+        "k_sweep_fwd": nc * (32 + 25 * t + 5 * t),
+        "k_sweep_bwd": nc * (32 + 25 * t + 5 * t),
+        # W, M, Lambda, velocity, SA diagonal in; record heads (2 x 13 T) and about four
         # stencil entries of 4 T out; face geometry and spectral radius
-        "k_sweep_prep": nc * (2 * 5 * 8 + 8 + 2 * 8 + 8 + 28 * t + 16 * t) + nf * (6 * 8),
+        "k_sweep_prep": nc * (2 * 5 * 8 + 8 + 2 * 8 + 8 + 26 * t + 16 * t) + nf * (6 * 8),
     }
     return per.get(kernel)
 
@@ -443,8 +446,8 @@ def rooflines(res, mesh, precision, workload, probe_tflops=None):
     peak, mhz = fp64_peak(res.get("clocks"))
     flux_t = km["k_flux"]
     ach_f = FLUX_ALG_FLOPS_PER_FACE * mesh.n_faces / (flux_t / 1e3) / 1e12
-    exe = ncu.get("flux_exec_flops_per_face")
-    dram = ncu.get("flux_dram_bytes_per_face")
+    exe = ncu.get("flux_exec_flops_per_face", {}).get(t)
+    dram = ncu.get("flux_dram_bytes_per_face", {}).get(t)
     flux = {"bound": "alu", "kernel": "k_flux", "achieved": ach_f, "peak": peak, "unit": "TFLOP/s",
             "frac": ach_f / peak, "traffic": dram * mesh.n_faces if dram else None,
             "peak_source": f"derived: {SM_COUNT} SMs x 2 FP64 FMA/clk x 2 flop x {mhz:.0f} MHz (median SM clock "
