@@ -546,10 +546,10 @@ __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int
 //    values are 48 or 96 bytes, which puts consecutive cells on distinct banks), SA apart.
 // Forward + backward on the 20,480-cell hybrid plate (351 levels each way), against one
 // thread per cell that read its record inside the level and stored its results itself:
-// FP32 401 + 418 -> 174 + 151 us, double-float 592 + 719 -> 344 + 316, FP64 1192 + 1417 ->
+// FP32 401 + 418 -> 172 + 147 us, double-float 592 + 719 -> 344 + 316, FP64 1192 + 1417 ->
 // 756 + 695 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
 // 60,160-cell O-mesh (605 levels; every level has a seam cell whose neighbour left the ring
-// 300 levels ago) FP32 946 + 895 -> 455 + 450 us; 5,003 cells of plate 160 + 188 -> 64 + 59.
+// 300 levels ago) FP32 946 + 895 -> 442 + 444 us; 5,003 cells of plate 160 + 188 -> 61 + 58.
 // A level ends when the store warps have stored the level before: one 16-byte store instead of
 // two of 8, and targets of two rounds read ahead instead of three, took FP32 forward from 184
 // and 492 to 176 and 457 us; a cell's increments side by side in dW (INC_STRIDE) took backward
@@ -611,8 +611,8 @@ __device__ __forceinline__ void bulk_g2s(unsigned dst, const void* src, unsigned
 // cluster, reads its records and what left the ring from global memory. CHUNK: an FP32
 // level takes 0.5 us, so the copies come in fewer, larger pieces.
 constexpr int LVL_SMEM = 2048;
-template <class T>
-constexpr int STORE_WARPS = sizeof(T) == 4 ? 3 : 2;
+// (three store warps in FP32: 1% slower, their shared-memory reads stand in the cells' way)
+constexpr int STORE_WARPS = 2;
 template <class T>
 struct Smem {
   static constexpr int SLOTS = ring_slots((int)sizeof(T)), ZERO = zero_slot((int)sizeof(T)), ALL = ZERO + 1;
@@ -1013,7 +1013,7 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
   const int pbase = glv[0], np = glv[nl] - pbase;
   const SweepRec<T>* grec = (const SweepRec<T>*)(FWD ? d.frec : d.brec) + pbase;
   const int tid = threadIdx.x;
-  constexpr int NST = 32 * STORE_WARPS<T>;
+  constexpr int NST = 32 * STORE_WARPS;
   const int nct = C == 1 ? (int)blockDim.x - NST - 64 : (int)blockDim.x;   // cell threads
   const int nbar = nct + NST + 32;                                 // threads of a level barrier
   const bool lvs = nl + 3 < LVL_SMEM;                              // level offsets in shared memory
@@ -1191,7 +1191,7 @@ constexpr int SETS = 2;
 template <class T>
 constexpr int SET_THREADS = sizeof(T) == 4 ? 224 : 192;
 template <class T>
-constexpr int block_threads(int set) { return SETS * set + 32 * STORE_WARPS<T> + 64; }
+constexpr int block_threads(int set) { return SETS * set + 32 * STORE_WARPS + 64; }
 template <class T, bool FWD>
 __global__ void __launch_bounds__(block_threads<T>(SET_THREADS<T>), 1)
 k_sweep_block(const __grid_constant__ Dev d) { sweep_narrow<T, FWD, 1, SETS>(d); }
