@@ -352,6 +352,23 @@ static int run_iterations(igks_ctx* ctx, int n) {
   return 0;
 }
 
+// cell -> faces in ascending face order
+static void cell_faces(const HostMesh& m, std::vector<int>& ptr, std::vector<int>& face) {
+  ptr.assign(m.nc + 1, 0);
+  for (int f = 0; f < m.nf; f++) {
+    ptr[m.face_cells[2 * f] + 1]++;
+    if (m.face_cells[2 * f + 1] >= 0) ptr[m.face_cells[2 * f + 1] + 1]++;
+  }
+  for (int i = 0; i < m.nc; i++) ptr[i + 1] += ptr[i];
+  face.assign(ptr[m.nc], 0);
+  std::vector<int> fill(m.nc, 0);
+  for (int f = 0; f < m.nf; f++) {
+    int l = m.face_cells[2 * f], r = m.face_cells[2 * f + 1];
+    face[ptr[l] + fill[l]++] = f;
+    if (r >= 0) face[ptr[r] + fill[r]++] = f;
+  }
+}
+
 // dependency levels of the sequential sweep: forward uses lower neighbours, backward upper
 static void sweep_levels(const HostMesh& m, const std::vector<int>& cf_ptr, const std::vector<int>& cf_face,
                          bool forward, std::vector<int>& order, std::vector<int>& lvl_ptr) {
@@ -383,6 +400,67 @@ static void sweep_levels(const HostMesh& m, const std::vector<int>& cf_ptr, cons
   }
 }
 
+// Narrow-schedule stencils of one direction in sweep-position order, all solves one after the
+// other: entries [ptr[p], ptr[p + 1]) of position p, their cells (-1 - face for a ghost) and
+// where the cell's increments are (SweepStat); per level the cells fetched into its side slots.
+struct SweepLists {
+  std::vector<int> ptr = std::vector<int>(1, 0), j, slot, side_ptr, side_j;
+};
+
+// Append a solve's stencils (cells from co, faces from fo on; map: cell-face entry -> list
+// entry, from cf0 on). Position q writes ring slot q % ring. A neighbour at position q is read
+// from its slot while the level ending at e is processed iff
+//  - q >= e - ring: nothing in the levels between the neighbour's and this one, nor in this
+//    one, maps to its slot, and
+//  - q - ring lies before the neighbour's own level: the cells of a level are worked on by
+//    several warps in no order, so of two positions of one level that share a slot (a level
+//    wider than the ring) either may be written last, and neither is read from the ring.
+static void sweep_stencil(const HostMesh& m, const std::vector<int>& lp, const std::vector<int>& lf, bool fwd,
+                          const std::vector<int>& ord, const std::vector<int>& lvl, int ring, int co, int fo, int cf0,
+                          SweepLists& o, std::vector<int>& map) {
+  std::vector<int> pos(m.nc), begin(m.nc);   // position of a cell, first position of its level
+  for (int l = 0; l + 1 < (int)lvl.size(); l++)
+    for (int p = lvl[l]; p < lvl[l + 1]; p++) { pos[ord[p]] = p; begin[ord[p]] = lvl[l]; }
+  const size_t side_max = o.side_j.size() + m.nc / 4;   // within the solve's footprint bound
+  for (int l = 0; l + 1 < (int)lvl.size(); l++) {
+    const int e = lvl[l + 1];
+    o.side_ptr.push_back((int)o.side_j.size());
+    for (int p = lvl[l]; p < e; p++) {
+      const int i = ord[p];
+      for (int k = lp[i]; k < lp[i + 1]; k++) {
+        const int f = lf[k];
+        const int l_ = m.face_cells[2 * f], r_ = m.face_cells[2 * f + 1];
+        if (r_ < 0) {
+          if (!fwd && (m.face_bc[f] == IGKS_BC_WALL || m.face_bc[f] == IGKS_BC_SYMMETRY ||
+                       m.face_bc[f] == IGKS_BC_MOVING_WALL)) {
+            map[cf0 + k] = (int)o.j.size();
+            o.j.push_back(-1 - (fo + f));
+            o.slot.push_back(SLOT_GHOST);
+          }
+          continue;
+        }
+        const int j = (l_ == i) ? r_ : l_;
+        if (fwd ? (j >= i) : (j <= i)) continue;
+        map[cf0 + k] = (int)o.j.size();
+        o.j.push_back(co + j);
+        // a neighbour that is not in the ring: its increments are fetched into one of the
+        // level's side slots, from two levels ahead on (they are in global memory by then)
+        const int q = pos[j];
+        int slot = SLOT_GLOBAL;
+        if (q >= e - ring && q - ring < begin[j]) slot = q % ring;
+        else if ((int)o.side_j.size() - o.side_ptr.back() < SIDE && o.side_j.size() < side_max && l >= 3 &&
+                 q < lvl[l - 2]) {
+          slot = ring + (l & 1) * SIDE + (int)o.side_j.size() - o.side_ptr.back();
+          o.side_j.push_back(co + j);
+        }
+        o.slot.push_back(slot);
+      }
+      o.ptr.push_back((int)o.j.size());
+    }
+  }
+  o.side_ptr.push_back((int)o.side_j.size());
+}
+
 static int build(igks_ctx* ctx) {
   if (ctx->built) return 0;
   if (ctx->meshes.empty()) return fail(ctx, IGKS_EINVAL, "no mesh uploaded");
@@ -405,10 +483,11 @@ static int build(igks_ctx* ctx) {
   std::vector<double> xy(2 * (size_t)nn);
   std::vector<int> fL(nf), fR(nf), fbc(nf), fsolve(nf), fnode(2 * (size_t)nf), bface, wall_face, wall_ptr(ns + 1, 0);
   std::vector<int> fwd_order, fwd_lvl, bwd_order, bwd_lvl, lsp(ns + 1, 0), blsp(ns + 1, 0);
-  std::vector<int> fs_ptr(1, 0), fs_j, fs_slot, cf_to_fs, bs_ptr(1, 0), bs_j, bs_slot, cf_to_bs;
+  SweepLists fs, bs;
+  std::vector<int> cf_to_fs, cf_to_bs;
   std::vector<SolveState> st(ns);
   std::vector<DevFlow> dfl(ns);
-  std::vector<int> gent_ptr(1, 0), gent_pos, fside_ptr, fside_j, bside_ptr, bside_j;
+  std::vector<int> gent_ptr(1, 0), gent_pos;
   const int tbytes = ctx->opt.precision == IGKS_PREC_MIXED ? 4 : 8;
   const int ring = ring_slots(tbytes), zslot = zero_slot(tbytes);
   for (int s = 0; s < ns; s++) {
@@ -418,22 +497,8 @@ static int build(igks_ctx* ctx) {
       xy[no + k] = m.xy[2 * k];
       xy[nn + no + k] = m.xy[2 * k + 1];
     }
-    // cell -> faces in ascending face order
-    std::vector<int> lp(m.nc + 1, 0), lf;
-    for (int f = 0; f < m.nf; f++) {
-      lp[m.face_cells[2 * f] + 1]++;
-      if (m.face_cells[2 * f + 1] >= 0) lp[m.face_cells[2 * f + 1] + 1]++;
-    }
-    for (int i = 0; i < m.nc; i++) lp[i + 1] += lp[i];
-    lf.assign(lp[m.nc], 0);
-    {
-      std::vector<int> fill(m.nc, 0);
-      for (int f = 0; f < m.nf; f++) {
-        int l = m.face_cells[2 * f], r = m.face_cells[2 * f + 1];
-        lf[lp[l] + fill[l]++] = f;
-        if (r >= 0) lf[lp[r] + fill[r]++] = f;
-      }
-    }
+    std::vector<int> lp, lf;
+    cell_faces(m, lp, lf);
     for (int i = 0; i < ctx->cell_pad[s]; i++) {
       int g = co + i;
       if (i < m.nc) {
@@ -470,62 +535,14 @@ static int build(igks_ctx* ctx) {
     for (int c : ord) bwd_order.push_back(co + c);
     for (int p : lvl) bwd_lvl.push_back(base + p);
     blsp[s + 1] = (int)bwd_lvl.size();
-    // narrow-schedule stencils in sweep-position order, with shared-memory ring slots: a
-    // neighbour produced at position q is still in the ring while the current level (end
-    // e) is processed iff q >= e - ring (no position written during the level maps to its
-    // slot)
+    // narrow-schedule stencils
     cf_to_fs.resize(cf_face.size(), -1);
     cf_to_bs.resize(cf_face.size(), -1);
     for (int dir = 0; dir < 2; dir++) {
       const bool fwd = dir == 0;
       std::vector<int> ordl, lvll;
       sweep_levels(m, lp, lf, fwd, ordl, lvll);
-      std::vector<int> pos(m.nc);
-      for (int p = 0; p < m.nc; p++) pos[ordl[p]] = p;
-      std::vector<int>& sptr = fwd ? fs_ptr : bs_ptr;
-      std::vector<int>& sj = fwd ? fs_j : bs_j;
-      std::vector<int>& sslot = fwd ? fs_slot : bs_slot;
-      std::vector<int>& map = fwd ? cf_to_fs : cf_to_bs;
-      std::vector<int>& side_ptr = fwd ? fside_ptr : bside_ptr;
-      std::vector<int>& side_j = fwd ? fside_j : bside_j;
-      const size_t side_max = side_j.size() + m.nc / 4;   // within the solve's footprint bound
-      for (int l = 0; l + 1 < (int)lvll.size(); l++) {
-        const int e = lvll[l + 1];
-        side_ptr.push_back((int)side_j.size());
-        for (int p = lvll[l]; p < e; p++) {
-          const int i = ordl[p];
-          for (int k = lp[i]; k < lp[i + 1]; k++) {
-            const int f = lf[k];
-            const int l_ = m.face_cells[2 * f], r_ = m.face_cells[2 * f + 1];
-            const int kg = cf_ptr[co + i] + (k - lp[i]);
-            if (r_ < 0) {
-              if (!fwd && (m.face_bc[f] == IGKS_BC_WALL || m.face_bc[f] == IGKS_BC_SYMMETRY ||
-                           m.face_bc[f] == IGKS_BC_MOVING_WALL)) {
-                map[kg] = (int)sj.size();
-                sj.push_back(-1 - (fo + f));
-                sslot.push_back(SLOT_GHOST);
-              }
-              continue;
-            }
-            const int j = (l_ == i) ? r_ : l_;
-            if (fwd ? (j >= i) : (j <= i)) continue;
-            map[kg] = (int)sj.size();
-            sj.push_back(co + j);
-            // a neighbour that left the ring: its increments are fetched into one of the
-            // level's side slots, from two levels ahead on (they are in global memory by then)
-            int slot = SLOT_GLOBAL;
-            if (pos[j] >= e - ring) slot = pos[j] % ring;
-            else if ((int)side_j.size() - side_ptr.back() < SIDE && side_j.size() < side_max && l >= 3 &&
-                     pos[j] < lvll[l - 2]) {
-              slot = ring + (l & 1) * SIDE + (int)side_j.size() - side_ptr.back();
-              side_j.push_back(co + j);
-            }
-            sslot.push_back(slot);
-          }
-          sptr.push_back((int)sj.size());
-        }
-      }
-      side_ptr.push_back((int)side_j.size());
+      sweep_stencil(m, lp, lf, fwd, ordl, lvll, ring, co, fo, cf_ptr[co], fwd ? fs : bs, fwd ? cf_to_fs : cf_to_bs);
     }
     // state
     SolveState& q = st[s];
@@ -555,9 +572,8 @@ static int build(igks_ctx* ctx) {
   }
   for (int dir = 0; dir < 2; dir++) {
     const bool fwd = dir == 0;
-    const std::vector<int>& sptr = fwd ? fs_ptr : bs_ptr;
-    const std::vector<int>& sj = fwd ? fs_j : bs_j;
-    const std::vector<int>& sslot = fwd ? fs_slot : bs_slot;
+    const SweepLists& lists = fwd ? fs : bs;
+    const std::vector<int>&sptr = lists.ptr, &sj = lists.j, &sslot = lists.slot;
     const std::vector<int>& map = fwd ? cf_to_fs : cf_to_bs;
     const std::vector<int>& pos = fwd ? pos_f : pos_b;
     std::vector<SweepStat>& rec = fwd ? fst : bst;
@@ -587,7 +603,7 @@ static int build(igks_ctx* ctx) {
   for (int s = 0, p = 0; s < ns; s++) {      // cells with ghosts in their backward records, per solve
     for (const int end = p + ctx->meshes[s].nc; p < end; p++) {
       bool ghost = false;
-      for (int k = bs_ptr[p]; k < bs_ptr[p + 1]; k++) ghost |= bs_slot[k] == SLOT_GHOST;
+      for (int k = bs.ptr[p]; k < bs.ptr[p + 1]; k++) ghost |= bs.slot[k] == SLOT_GHOST;
       if (ghost && !(bst[p].kind & KIND_CSR)) gent_pos.push_back(p);
     }
     gent_ptr.push_back((int)gent_pos.size());
@@ -627,10 +643,10 @@ static int build(igks_ctx* ctx) {
   d.starve_test = ctx->opt.starve_test;
   d.nnz = (int)cf_face.size();
   AL(sw_cell, double, 5 * (size_t)nc); AL(sw_st, double, std::max(4 * (size_t)d.nnz, 8 * (size_t)nc)); AL(sw_j, int, d.nnz);
-  UP(fs_ptr, fs_ptr); UP(fs_j, fs_j); UP(fs_slot, fs_slot); UP(cf_to_fs, cf_to_fs);
-  UP(bs_ptr, bs_ptr); UP(bs_j, bs_j); UP(bs_slot, bs_slot); UP(cf_to_bs, cf_to_bs);
-  d.nfs = (int)fs_j.size();
-  d.nbs = (int)bs_j.size();
+  UP(fs_ptr, fs.ptr); UP(fs_j, fs.j); UP(fs_slot, fs.slot); UP(cf_to_fs, cf_to_fs);
+  UP(bs_ptr, bs.ptr); UP(bs_j, bs.j); UP(bs_slot, bs.slot); UP(cf_to_bs, cf_to_bs);
+  d.nfs = (int)fs.j.size();
+  d.nbs = (int)bs.j.size();
   AL(sc_f, double, 4 * (size_t)std::max(d.nfs, 1)); AL(sc_b, double, 4 * (size_t)std::max(d.nbs, 1));
   d.npos = P;
   UP(pos_f, pos_f); UP(pos_b, pos_b);
@@ -641,7 +657,7 @@ static int build(igks_ctx* ctx) {
   CK(h2d_2d(ctx, d.frec, rec, fst.data(), sizeof(SweepStat), sizeof(SweepStat), P));
   CK(h2d_2d(ctx, d.brec, rec, bst.data(), sizeof(SweepStat), sizeof(SweepStat), P));
   UP(fj, fj); UP(bj, bj);
-  UP(fside_ptr, fside_ptr); UP(fside_j, fside_j); UP(bside_ptr, bside_ptr); UP(bside_j, bside_j);
+  UP(fside_ptr, fs.side_ptr); UP(fside_j, fs.side_j); UP(bside_ptr, bs.side_ptr); UP(bside_j, bs.side_j);
   UP(gent_ptr, gent_ptr); UP(gent_pos, gent_pos);
   d.ring = ring;
   AL(gprim, double, 6 * (size_t)nf);
@@ -1238,6 +1254,32 @@ int igks_order_cells(int32_t n_cells, int32_t n_faces, const int32_t* face_cells
   for (int c = 0; c < nc; c++) cnt[c + 1] += cnt[c];
   for (int i = 0; i < n_cells; i++) perm[cnt[col[i]]++] = i;
   if (n_colors) *n_colors = nc;
+  return IGKS_OK;
+}
+
+// Test hook (host only, not part of the ABI): the narrow schedule of one mesh. lvl [n_cells + 1]
+// receives the level offsets (*n_levels + 1 of them), order [n_cells] the cell at each position,
+// ptr [n_cells + 1], j and slot [2 n_faces] the stencil entries, *ring the ring's slots.
+int igks_sweep_schedule_(int32_t n_cells, int32_t n_faces, const int32_t* face_cells, const int32_t* face_bc,
+                         int32_t precision, int32_t forward, int32_t* lvl, int32_t* n_levels, int32_t* order,
+                         int32_t* ptr, int32_t* j, int32_t* slot, int32_t* ring) {
+  HostMesh m;
+  m.nc = n_cells; m.nf = n_faces;
+  m.face_cells.assign(face_cells, face_cells + 2 * (size_t)n_faces);
+  m.face_bc.assign(face_bc, face_bc + n_faces);
+  std::vector<int> lp, lf, ord, lv;
+  cell_faces(m, lp, lf);
+  sweep_levels(m, lp, lf, forward != 0, ord, lv);
+  SweepLists o;
+  std::vector<int> map(lf.size(), -1);
+  *ring = ring_slots(precision == IGKS_PREC_MIXED ? 4 : 8);
+  sweep_stencil(m, lp, lf, forward != 0, ord, lv, *ring, 0, 0, 0, o, map);
+  *n_levels = (int)lv.size() - 1;
+  std::copy(lv.begin(), lv.end(), lvl);
+  std::copy(ord.begin(), ord.end(), order);
+  std::copy(o.ptr.begin(), o.ptr.end(), ptr);
+  std::copy(o.j.begin(), o.j.end(), j);
+  std::copy(o.slot.begin(), o.slot.end(), slot);
   return IGKS_OK;
 }
 
