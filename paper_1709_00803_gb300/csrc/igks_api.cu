@@ -663,7 +663,7 @@ static int build(igks_ctx* ctx) {
   AL(gprim, double, 6 * (size_t)nf);
   d.lgrad = (double*)d.sw_st;
   setup_sweeps();
-  CK(flux_table_init());
+  if (ctx->opt.precision != IGKS_PREC_MIXED) CK(upload_flux_table(ctx->stream));
   {
     // wide schedule: level l of every solve, solves in order
     int maxf = 0, maxb = 0;

@@ -203,7 +203,7 @@ void launch_init_state(const Dev& d, int solve, cudaStream_t s);
 void launch_prep(const Dev& d, cudaStream_t s);
 void launch_ghost(const Dev& d, cudaStream_t s);
 void launch_gradient(const Dev& d, cudaStream_t s);
-cudaError_t flux_table_init();   // the flux's device table, once per device (current device)
+cudaError_t upload_flux_table(cudaStream_t s);   // the table of the FP64 and double-float solves' flux
 void launch_flux(const Dev& d, int precision, cudaStream_t s);
 void launch_residual(const Dev& d, cudaStream_t s);
 void launch_norms(const Dev& d, cudaStream_t s);

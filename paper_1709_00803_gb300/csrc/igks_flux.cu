@@ -13,7 +13,6 @@
 // Two kernels: k_flux (igks_gks.cuh) for FP64 and double-float sweeps, k_flux_moment
 // (igks_gks_moment.cuh) for mixed precision, whose iterates keep their bits.
 #include <cmath>
-#include <mutex>
 #include <vector>
 
 #include "igks_dev.h"
@@ -269,13 +268,7 @@ __global__ void __launch_bounds__(128, 1) k_flux_moment(Dev d) {
 
 // The nodes of gks::normal_tail in extended precision: c_0 = Q(z), c_(n+1) =
 // (-1)^(n+1) He_n(z) phi(z) / (n + 1)!, He_(n+1) = z He_n - n He_(n-1).
-cudaError_t flux_table_init() {
-  static std::mutex mu;
-  static bool done[64] = {};
-  std::lock_guard<std::mutex> lock(mu);
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess || (dev < 64 && done[dev])) return e;
+static std::vector<double> tail_table() {
   std::vector<double> t(8 * (size_t)gks::TAIL_NODES, 0.0);
   for (int k = 0; k < gks::TAIL_NODES; k++) {
     const long double z = (long double)k / gks::TAIL_PER_UNIT;
@@ -292,9 +285,15 @@ cudaError_t flux_table_init() {
       h1 = h2;
     }
   }
-  e = cudaMemcpyToSymbol(gks::g_tail, t.data(), t.size() * sizeof(double));
-  if (e == cudaSuccess && dev < 64) done[dev] = true;
-  return e;
+  return t;
+}
+
+// Every context uploads the table on its own stream, ahead of its kernels (192 KiB, always
+// the same bytes): nothing is assumed about what other contexts, streams or a device reset
+// before have left in it. Only the host's copy is kept.
+cudaError_t upload_flux_table(cudaStream_t s) {
+  static const std::vector<double> t = tail_table();
+  return cudaMemcpyToSymbolAsync(gks::g_tail, t.data(), t.size() * sizeof(double), 0, cudaMemcpyHostToDevice, s);
 }
 
 void launch_flux(const Dev& d, int precision, cudaStream_t s) {

@@ -37,7 +37,7 @@ static_assert(KDOF == 3, "the moments over v and xi below are written for K = 3"
 // ---- normal tail and density ----
 // Node k at z = k / 512: Taylor coefficients of Q(z) = P(N(0,1) > z), degree 6 (|t| <= 2^-10:
 // the remainder is below 1e-16 of Q, and of the density -Q', up to z = 6). 64 bytes a node,
-// 192 KiB, computed by the host in extended precision (flux_table_init).
+// 192 KiB, computed by the host in extended precision (upload_flux_table).
 constexpr int TAIL_PER_UNIT = 512, TAIL_MAX = 6, TAIL_NODES = TAIL_PER_UNIT * TAIL_MAX + 1;
 static __device__ __align__(64) double g_tail[TAIL_NODES * 8];
 
