@@ -583,7 +583,12 @@ static int build(igks_ctx* ctx) {
     for (size_t k = 0; k < map.size(); k++)
       if (map[k] >= 0) inv[map[k]] = (int)k;
     for (size_t k = 0; k < sj.size(); k++)   // cells whose increments are read from global memory
-      if (sslot[k] == SLOT_GLOBAL || sslot[k] >= ring) rec[pos[sj[k]]].spill = 1;
+      if (sslot[k] == SLOT_GLOBAL || sslot[k] >= ring) rec[pos[sj[k]]].spill = SPILL_READ;
+    const std::vector<int>&lvl = fwd ? fwd_lvl : bwd_lvl, &first = fwd ? lsp : blsp;
+    for (int s = 0; s < ns; s++)             // levels whose slots the next one takes again
+      for (int l = first[s]; l + 1 < first[s + 1]; l++)
+        if (lvl[std::min(l + 2, first[s + 1] - 1)] - lvl[l] > ring)
+          for (int p = lvl[l]; p < lvl[l + 1]; p++) rec[p].spill |= SPILL_OWN;
     for (int p = 0; p < P; p++) {
       SweepStat& q = rec[p];
       int q0 = sptr[p];

@@ -43,8 +43,8 @@ constexpr int PF_E = 3;              // stencil entries held per sweep record
 // Records of the narrow sweeps, one per sweep position and direction, brought into shared
 // memory by bulk copies.
 // Static part (uploaded once): cell, kind (entry count, and the flags below), the cell's
-// backward position (forward records), whether a later cell reads this cell's increments
-// from global memory, and per entry where the neighbour's increments are: a slot of the
+// backward position (forward records), what the cell itself stores to global memory (spill,
+// the flags below), and per entry where the neighbour's increments are: a slot of the
 // shared-memory ring, from ring_slots on a side slot (a neighbour that left the ring,
 // fetched again ahead of its level), ZERO_SLOT (no entry: reads zeros, and its coefficients
 // stay zero), SLOT_GLOBAL (read from global memory) or SLOT_GHOST (a wall or symmetry ghost
@@ -64,6 +64,8 @@ constexpr int KIND_THIRD = 8;        // a third entry, all three in ring or side
 constexpr int KIND_RARE = 16;        // a ghost, or a neighbour in global memory
 constexpr int KIND_SIDE = 32;        // a side slot (used by staged solves only)
 constexpr int KIND_CSR = 64;         // more than PF_E entries: the CSR stencil (KIND_RARE too)
+constexpr int SPILL_READ = 1;        // a later cell reads this cell's increments from global memory
+constexpr int SPILL_OWN = 2;         // the level and the next do not fit the ring: no store warp takes it
 struct alignas(16) SweepStat { int i, kind, pb, spill; int slot[PF_E], pad; };
 struct alignas(16) SweepJ { int j[PF_E], pad; };            // the entries' cells, -1 - face for a ghost
 template <class T>

@@ -607,9 +607,9 @@ __device__ __forceinline__ void bulk_g2s(unsigned dst, const void* src, unsigned
 
 // shared memory: ring, side slots and the zero slot [12] | their SA increments | NREC records
 // | LVL_SMEM level offsets | an mbarrier per chunk | progress: levels finished | landed:
-// records in shared memory. A solve with a level wider than NREC - CHUNK positions, or a
-// cluster, reads its records and what left the ring from global memory. CHUNK: an FP32
-// level takes 0.5 us, so the copies come in fewer, larger pieces.
+// records in shared memory. Records that find no place in a level wider than NREC - CHUNK
+// positions, and all of a cluster's, are read from global memory. CHUNK: an FP32 level takes
+// 0.5 us, so the copies come in fewer, larger pieces.
 constexpr int LVL_SMEM = 2048;
 // (three store warps in FP32: 1% slower, their shared-memory reads stand in the cells' way)
 constexpr int STORE_WARPS = 2;
@@ -625,7 +625,7 @@ struct Smem {
   static constexpr size_t bar = lvl + (size_t)LVL_SMEM * sizeof(int);
   static constexpr size_t flag = bar + 8 * (size_t)NCHUNK;
   static constexpr size_t total = flag + 16;
-  static_assert(2 * (NREC - CHUNK) <= SLOTS, "two staged levels fit the ring");
+  static_assert(NCHUNK <= 32, "a phase bit per buffer");
   static_assert(total <= 232448, "shared memory of one block");
 };
 
@@ -766,15 +766,25 @@ __device__ __forceinline__ void store_inc(const Dev& d, int at, const T* w, T w4
   }
 }
 
-// the increments of a cell that a later one reads from global memory (before the barrier)
+// what a cell thread itself stores (before the barrier): the increments and flux increments that
+// a later cell reads from global memory (SPILL_READ), and the increments of a level that the
+// store warps do not take (SPILL_OWN; pb: the cell's backward position)
 template <class T, bool FWD>
-__device__ __noinline__ void store_spill(const Dev& d, int i, LaneOut<T> o, int lane) {
+__device__ __noinline__ void store_spill(const Dev& d, int i, int pb, int spill, LaneOut<T> o, int lane) {
   const int n = d.nc_pad;
+  if (FWD && (spill & SPILL_OWN)) {
+    T* m = ((SweepRec<T>*)d.brec + pb)->m;
+    m[2 * lane] = o.w0;
+    m[2 * lane + 1] = o.w1;
+    if (lane) m[4] = o.w4;
+  }
+  if (FWD && !(spill & SPILL_READ)) return;
   T* dWv = (T*)(FWD ? d.dWs : d.dW);
   T* dF = (T*)d.dF;
   dWv[inc_at<T>(n, 2 * lane, i)] = o.w0;
   dWv[inc_at<T>(n, 2 * lane + 1, i)] = o.w1;
   if (lane) dWv[inc_at<T>(n, 4, i)] = o.w4;
+  if (!(spill & SPILL_READ)) return;
   for (int v = 0; v < 4; v++) dF[(2 * v + lane) * n + i] = o.f[v];
 }
 
@@ -857,7 +867,7 @@ __device__ __forceinline__ RingAt ring_at(const LaneRec<T>& rc, int q, int lane)
 }
 
 // The increments of the cell at position p (its record in rc). rare: the kinds that take the
-// general path (with the side slots' when the solve is not staged). co2(): the third entry's
+// general path (with the side slots' in a cluster). co2(): the third entry's
 // coefficients in memory. Called by whole warps; a thread without a cell of its own (valid =
 // false) works on a copy of another's and stores nothing.
 template <class T, bool FWD, int C, class Co2>
@@ -904,7 +914,8 @@ __device__ __forceinline__ LaneOut<T> lane_cell(const Dev& d, T* ring, T* ring4,
   const LaneOut<T> o = lane_finish<T, FWD>(rc, acc0, acc1, acc4, lane, sa_on);
   if (valid) {
     ring_put<T>(ring + at.put, ring4 + at.put4, o, lane);
-    if (rc.spill) store_spill<T, FWD>(d, rc.i, o, lane);
+    const int spill = C == 1 ? rc.spill : rc.spill & SPILL_READ;   // (a cluster's cells store all the same)
+    if (spill) store_spill<T, FWD>(d, rc.i, rc.pb, spill, o, lane);
   }
   return o;
 }
@@ -979,12 +990,14 @@ __device__ __forceinline__ void st_release(int* p, int v) {
 //    set reads its next records (from shared memory as far as they have landed, the others
 //    from global memory) before it waits for the level before, so with two sets nothing but
 //    the ring reads, the arithmetic and the ring stores lies between two levels;
-//  - store warps: the increments of level k to global memory during level k + 1 (their ring
-//    slots are not reused before level k + 2: two levels fit the ring);
+//  - store warps: the increments of level k to global memory during level k + 1, if the two
+//    levels fit the ring together (their slots are then not reused before level k + 2); the
+//    cell warps store wider levels themselves;
 //  - the side warp fetches increments that left the ring: it reads them during level k for
 //    level k + 2 and puts them into the side slots during level k + 1;
 //  - the copy warp: a chunk's buffer is free once all its positions lie in finished levels;
-//    it issues chunks as buffers become free and counts the records that have landed. It
+//    it issues chunks as buffers become free and counts the records that have landed (chunks of
+//    a level wider than the buffers that it has finished without are passed over). It
 //    runs beside the level barriers, and nobody waits for it. A chunk that has not landed
 //    after wait_limit tries marks the solve IGKS_TIMEOUT (the update leaves its state
 //    untouched); the warp then waits for the other copies in flight and ends.
@@ -1017,24 +1030,19 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
   const int nct = C == 1 ? (int)blockDim.x - NST - 64 : (int)blockDim.x;   // cell threads
   const int nbar = nct + NST + 32;                                 // threads of a level barrier
   const bool lvs = nl + 3 < LVL_SMEM;                              // level offsets in shared memory
-  int wide = 0;
-  for (int k = tid; k <= nl + 2; k += blockDim.x) {
-    const int v = glv[min(k, nl)] - pbase;
-    if (lvs) slv[k] = v;
-    if (k > 0) wide |= (v - (glv[min(k - 1, nl)] - pbase)) > S::NREC - S::CHUNK;
-  }
+  if (lvs)
+    for (int k = tid; k <= nl + 2; k += blockDim.x) slv[k] = glv[min(k, nl)] - pbase;
   if (C == 1 && tid < S::NCHUNK) mbar_init(bar0 + 8 * tid, 1);
   if (C == 1) asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   if (tid == 0) { *progress = 0; *landed_p = 0; }
   if (tid < 13) (tid < 12 ? ring + 12 * S::ZERO : ring4 + S::ZERO - 12)[tid] = (T)0;
-  const bool staged = !__syncthreads_or(wide) && C == 1;
+  __syncthreads();
   if constexpr (C > 1) cg::this_cluster().sync();                  // every block runs before any remote read
   auto lv = [&](int k) { return lvs ? slv[k] : glv[min(k, nl)] - pbase; };
-
   if (tid < nct) {
     const int set = tid / (nct / SETS), t = tid - set * (nct / SETS);
     const int lane = t & 1, w0 = (t & 31) / 2 * C, own = C * (t >> 1), step = C * (nct / SETS) / 2;
-    const int rare = staged ? KIND_RARE : KIND_RARE | KIND_SIDE;
+    constexpr int rare = C == 1 ? KIND_RARE : KIND_RARE | KIND_SIDE;   // (no side warp in a cluster)
     LaneRec<T> rc;
     auto fetch = [&](int q, int landed) {
       if (q < landed) load_rec<T, FWD>(rc, srec + q % S::NREC, lane);
@@ -1052,19 +1060,19 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
       const bool act = q - w0 < e;       // a warp works if its first cell exists
       if (act) next();
       if (C == 1 && k > 0) bar_wait(2 - (k & 1), nbar);            // level k - 1 is finished
-      bool global = !staged;             // increments stored to global memory that others may read
+      bool global = false;               // increments stored to global memory that others may read
       if (act) do {                      // more than one round in a level wider than the set
         const bool valid = q < e;
         const int qc = min(q, e - 1);
         const LaneOut<T> o = lane_cell<T, FWD, C>(
             d, ring, ring4, rare, rc, at, pbase + qc, lane, valid, sa_on,
             [&] { return qc < landed ? srec[qc % S::NREC].co[2] : grec[qc].co[2]; });
-        if (C > 1 || !staged) {          // no store warps, or levels that may overrun the ring
+        if constexpr (C > 1) {           // no store warps
           const T p0 = shfl_pair(o.w0), p1 = shfl_pair(o.w1);
           const T w[4] = {o.w0, o.w1, p0, p1};
           if (valid && lane == 0) store_inc<T, FWD>(d, FWD ? rc.pb : rc.i, w, o.w4);
         }
-        global |= rc.spill != 0;
+        global |= (rc.spill & SPILL_READ) != 0;
         q += step;
         if (q - w0 >= e) break;
         next();
@@ -1083,22 +1091,22 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
 #pragma unroll
     for (int j = 0; j < ROUNDS; j++) next[j] = t + j * NST < en ? at(t + j * NST) : 0;
     for (int k = 0; k <= nl; k++) {                                // stores level k - 1
-      if (staged) {
-        if (t == 0) st_release(progress, k);                       // levels below k are finished
-        auto put = [&](int q, int x) {
-          const int slot = q & (S::SLOTS - 1);
-          alignas(16) T w[4];
-          load_co<T>(w, ring + slot * 12 + 8);
-          store_inc<T, FWD>(d, x, w, ring4[slot]);
-        };
+      if (t == 0) st_release(progress, k);                         // levels below k are finished
+      const bool mine = en - b <= S::SLOTS;                        // (else SPILL_OWN)
+      auto put = [&](int q, int x) {
+        const int slot = q & (S::SLOTS - 1);
+        alignas(16) T w[4];
+        load_co<T>(w, ring + slot * 12 + 8);
+        store_inc<T, FWD>(d, x, w, ring4[slot]);
+      };
 #pragma unroll
-        for (int j = 0; j < ROUNDS; j++) {
-          const int x = next[j];
-          if (e + t + j * NST < en) next[j] = at(e + t + j * NST);
-          if (b + t + j * NST < e) put(b + t + j * NST, x);
-        }
-        for (int q = b + t + ROUNDS * NST; q < e; q += NST) put(q, at(q));
+      for (int j = 0; j < ROUNDS; j++) {
+        const int x = next[j];
+        if (e + t + j * NST < en) next[j] = at(e + t + j * NST);
+        if (mine && b + t + j * NST < e) put(b + t + j * NST, x);
       }
+      if (mine)
+        for (int q = b + t + ROUNDS * NST; q < e; q += NST) put(q, at(q));
       if (k == nl) break;
       bar_wait(1 + (k & 1), nbar);
       b = e; e = en; en = lv(k + 2);
@@ -1113,43 +1121,49 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
     // side slots, a step a level: offsets (level k + 4), cell (k + 3), increments (k + 2), slot (k + 1)
     int pa = 0, pb = 0, j = -1, jv = -1;
     T v[13];
-    if (staged && nl > 3) { pa = sp[3]; pb = sp[4]; }
+    if (nl > 3) { pa = sp[3]; pb = sp[4]; }
     for (int k = 0; k < nl; k++) {
-      if (staged) {
-        if (jv >= 0) {
-          const int slot = S::SLOTS + ((k + 1) & 1) * SIDE + t;
+      if (jv >= 0) {
+        const int slot = S::SLOTS + ((k + 1) & 1) * SIDE + t;
 #pragma unroll
-          for (int c = 0; c < 12; c++) ring[slot * 12 + c] = v[c];
-          ring4[slot] = v[12];
-        }
-        jv = j;
-        if (jv >= 0) {
-#pragma unroll
-          for (int c = 0; c < 4; c++) {
-            v[c] = dF[2 * c * n + jv];
-            v[4 + c] = dF[(2 * c + 1) * n + jv];
-            v[8 + c] = dWv[inc_at<T>(n, c, jv)];
-          }
-          v[12] = dWv[inc_at<T>(n, 4, jv)];
-        }
-        j = pa + t < pb ? sj[pa + t] : -1;
-        if (k + 5 <= nl) { pa = sp[k + 4]; pb = sp[k + 5]; }
-        else pa = pb;
+        for (int c = 0; c < 12; c++) ring[slot * 12 + c] = v[c];
+        ring4[slot] = v[12];
       }
+      jv = j;
+      if (jv >= 0) {
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          v[c] = dF[2 * c * n + jv];
+          v[4 + c] = dF[(2 * c + 1) * n + jv];
+          v[8 + c] = dWv[inc_at<T>(n, c, jv)];
+        }
+        v[12] = dWv[inc_at<T>(n, 4, jv)];
+      }
+      j = pa + t < pb ? sj[pa + t] : -1;
+      if (k + 5 <= nl) { pa = sp[k + 4]; pb = sp[k + 5]; }
+      else pa = pb;
       bar_wait(1 + (k & 1), nbar);
     }
-  } else if (staged && (tid & 31) == 0) {
+  } else if ((tid & 31) == 0) {
     constexpr int CHUNK = S::CHUNK;
     const int nchunk = (np + CHUNK - 1) / CHUNK;
     const unsigned urec = (unsigned)__cvta_generic_to_shared(smem_raw + S::rec);
     int issued = 0, landed = 0, seen = -1, idle = 0;
+    unsigned phase = 0;                                            // of each buffer's mbarrier
+    auto wait = [&](int q) {
+      const int c = q % S::NCHUNK;
+      const bool ok = mbar_wait(bar0 + 8 * c, phase >> c & 1, d.wait_limit);
+      phase ^= 1u << c;
+      return ok;
+    };
     while (landed < nchunk && idle < d.wait_limit) {
       const int k = ld_acquire(progress);
       idle = k == seen ? idle + 1 : 0;
       if (k != seen) {
         seen = k;
         if (k >= nl) break;                                        // the sweep is over
-        const int upto = min(lv(k) / CHUNK + S::NCHUNK, nchunk);
+        const int first = lv(k) / CHUNK, upto = min(first + S::NCHUNK, nchunk);
+        if (landed == issued && first > issued) issued = landed = first;   // finished from global memory
         // the buffers were read by generic loads: order those before the async proxy's writes
         if (issued < upto) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         for (; issued < upto; issued++) {
@@ -1163,7 +1177,7 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
         }
       }
       if (landed < issued) {
-        if (!mbar_wait(bar0 + 8 * (landed % S::NCHUNK), (unsigned)((landed / S::NCHUNK) & 1), d.wait_limit)) {
+        if (!wait(landed)) {
           d.tmo[s] = 1;
           landed++;                                                // the others in flight land below
           break;
@@ -1175,8 +1189,7 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
       }
     }
     for (; landed < issued; landed++)                              // let the copies in flight land
-      if (!(FWD && d.starve_test && landed == 1))
-        mbar_wait(bar0 + 8 * (landed % S::NCHUNK), (unsigned)((landed / S::NCHUNK) & 1), d.wait_limit);
+      if (!(FWD && d.starve_test && landed == 1)) wait(landed);
   }
   if constexpr (FWD) {
     if constexpr (C == 1) __syncthreads();                         // the increments stored above
