@@ -159,9 +159,7 @@ static int upload(igks_ctx* ctx, const T** out, const std::vector<T>& h) {
   return 0;
 }
 
-// the per-group streams, graphs and events (group 0's stream is the context stream when
-// there is one group)
-static void release_groups(igks_ctx* ctx) {
+static void release_graphs(igks_ctx* ctx) {
   if (ctx->bexec) cudaGraphExecDestroy(ctx->bexec);
   if (ctx->bgraph) cudaGraphDestroy(ctx->bgraph);
   ctx->bexec = nullptr;
@@ -171,6 +169,12 @@ static void release_groups(igks_ctx* ctx) {
   for (auto& g : ctx->ggraph) if (g) cudaGraphDestroy(g);
   ctx->ggexec.clear();
   ctx->ggraph.clear();
+}
+
+// the per-group streams, graphs and events (group 0's stream is the context stream when
+// there is one group)
+static void release_groups(igks_ctx* ctx) {
+  release_graphs(ctx);
   for (auto& evs : ctx->gev)
     for (auto e : evs) if (e) cudaEventDestroy(e);
   ctx->gev.clear();
@@ -239,9 +243,48 @@ static int group_sweeps(const igks_ctx* ctx, int s0, int s1) {
   return 0;
 }
 
+// One iteration of every group as a graph, and check_every iterations of the batch as one.
+static int capture_graphs(igks_ctx* ctx) {
+  const int G = ctx->n_groups;
+  ctx->ggraph.assign(G, nullptr);
+  ctx->ggexec.assign(G, nullptr);
+  if (ctx->opt.use_graph) {
+    for (int g = 0; g < G; g++) {
+      CK(cudaStreamBeginCapture(ctx->gstream[g], cudaStreamCaptureModeThreadLocal));
+      enqueue_iteration(ctx, g);
+      cudaError_t e = cudaStreamEndCapture(ctx->gstream[g], &ctx->ggraph[g]);
+      if (e != cudaSuccess) return fail(ctx, IGKS_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+      CK(cudaGraphInstantiate(&ctx->ggexec[g], ctx->ggraph[g], 0));
+    }
+    // the batch graph: check_every iterations of every group, the groups' chains running
+    // side by side (a group may run ahead of another inside it, as with the per-group
+    // launches); not with per-kernel timing, whose events must stay one per kernel
+    const int R = ctx->opt.check_every;
+    if (!ctx->opt.timing && R >= 2 && R <= MAX_BATCH_GRAPH_ITERS) {
+      CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
+      if (G > 1) {
+        cudaEventRecord(ctx->fork_ev, ctx->stream);
+        for (int g = 0; g < G; g++) cudaStreamWaitEvent(ctx->gstream[g], ctx->fork_ev, 0);
+      }
+      for (int g = 0; g < G; g++)
+        for (int r = 0; r < R; r++) enqueue_iteration(ctx, g);
+      if (G > 1)
+        for (int g = 0; g < G; g++) {
+          cudaEventRecord(ctx->join_ev[g], ctx->gstream[g]);
+          cudaStreamWaitEvent(ctx->stream, ctx->join_ev[g], 0);
+        }
+      cudaError_t e = cudaStreamEndCapture(ctx->stream, &ctx->bgraph);
+      if (e != cudaSuccess) return fail(ctx, IGKS_ECUDA, std::string("batch graph capture: ") + cudaGetErrorString(e));
+      CK(cudaGraphInstantiate(&ctx->bexec, ctx->bgraph, 0));
+      ctx->bgraph_iters = R;
+    }
+  }
+  return 0;
+}
+
 // Split the solves into groups of consecutive solves with about equal cell counts (one
 // group with the wide schedule, whose per-level launches span all solves), give each its
-// launch ranges, a stream and timing events, and capture one iteration of each as a graph.
+// launch ranges, a stream and timing events, and capture their graphs.
 static int setup_groups(igks_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   for (auto st : ctx->gstream) if (st) cudaStreamSynchronize(st);
@@ -286,40 +329,7 @@ static int setup_groups(igks_ctx* ctx) {
     ctx->join_ev.push_back(j);
   }
   if (G > 1) CK(cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming));
-  ctx->ggraph.assign(G, nullptr);
-  ctx->ggexec.assign(G, nullptr);
-  if (ctx->opt.use_graph) {
-    for (int g = 0; g < G; g++) {
-      CK(cudaStreamBeginCapture(ctx->gstream[g], cudaStreamCaptureModeThreadLocal));
-      enqueue_iteration(ctx, g);
-      cudaError_t e = cudaStreamEndCapture(ctx->gstream[g], &ctx->ggraph[g]);
-      if (e != cudaSuccess) return fail(ctx, IGKS_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-      CK(cudaGraphInstantiate(&ctx->ggexec[g], ctx->ggraph[g], 0));
-    }
-    // the batch graph: check_every iterations of every group, the groups' chains running
-    // side by side (a group may run ahead of another inside it, as with the per-group
-    // launches); not with per-kernel timing, whose events must stay one per kernel
-    const int R = ctx->opt.check_every;
-    if (!ctx->opt.timing && R >= 2 && R <= MAX_BATCH_GRAPH_ITERS) {
-      CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-      if (G > 1) {
-        cudaEventRecord(ctx->fork_ev, ctx->stream);
-        for (int g = 0; g < G; g++) cudaStreamWaitEvent(ctx->gstream[g], ctx->fork_ev, 0);
-      }
-      for (int g = 0; g < G; g++)
-        for (int r = 0; r < R; r++) enqueue_iteration(ctx, g);
-      if (G > 1)
-        for (int g = 0; g < G; g++) {
-          cudaEventRecord(ctx->join_ev[g], ctx->gstream[g]);
-          cudaStreamWaitEvent(ctx->stream, ctx->join_ev[g], 0);
-        }
-      cudaError_t e = cudaStreamEndCapture(ctx->stream, &ctx->bgraph);
-      if (e != cudaSuccess) return fail(ctx, IGKS_ECUDA, std::string("batch graph capture: ") + cudaGetErrorString(e));
-      CK(cudaGraphInstantiate(&ctx->bexec, ctx->bgraph, 0));
-      ctx->bgraph_iters = R;
-    }
-  }
-  return 0;
+  return capture_graphs(ctx);
 }
 
 // n iterations of every group, stream-ordered after the work already on the context stream
@@ -891,14 +901,22 @@ int igks_mesh_upload(igks_ctx* ctx, int32_t n_nodes, const double* xy, int32_t n
 int igks_set_flow(igks_ctx* ctx, int32_t solve, const igks_flow* f) {
   if (!ctx || !f || solve < 0 || solve >= (int)ctx->meshes.size()) return IGKS_EINVAL;
   if (!igks_check_flow_(f)) return fail(ctx, IGKS_EINVAL, "invalid flow conditions");
-  const bool other = ctx->built && ctx->flows[solve].scheme != f->scheme;
   ctx->flows[solve] = *f;
   ctx->flow_set[solve] = 1;
   if (ctx->built) {
     DevFlow d = make_devflow(*f);
     CK(h2d(ctx, (DevFlow*)ctx->dev.flow + solve, &d, sizeof d));
     CK(cudaStreamSynchronize(ctx->stream));
-    if (other) return setup_groups(ctx);   // its launches may change (group_sweeps)
+    bool other = false;   // the launches change with the scheme
+    for (Dev& g : ctx->gdev) {
+      const int sweeps = group_sweeps(ctx, g.g_solve0, g.g_solve0 + g.g_nsolve);
+      other |= g.sweeps != sweeps;
+      g.sweeps = sweeps;
+    }
+    if (other) {
+      release_graphs(ctx);   // (no iteration is under way on any stream)
+      return capture_graphs(ctx);
+    }
   }
   return IGKS_OK;
 }
