@@ -75,8 +75,10 @@ typedef struct igks_options {
   int32_t use_graph;      /* capture one iteration (per group) as a CUDA graph and replay it;
                              with 2 <= check_every <= 64 and no timing, also check_every
                              iterations of every group as one graph, launched once per check */
-  int32_t sweep_threads;  /* cell threads per block of the sweep kernels, two for each cell of a level
-                             (0: default; at most 256) */
+  int32_t sweep_threads;  /* cell threads of the sweep kernels, two for each cell of a level (0: default;
+                             at most 256): of a block of a cluster, or of each of the two sets that
+                             take turns in a one-block sweep, which hold at most 224 (mixed
+                             precision) or 192 */
   int32_t timing;         /* record CUDA events around every kernel (igks_kernel_times) */
   int32_t sweep_mode;     /* 0 automatic, 1 one block per solve walking its levels,
                              2 one launch per level over all solves (low-depth orderings) */
@@ -246,8 +248,8 @@ int igks_get_forces(igks_ctx* ctx, int32_t solve, int32_t bc_tag, double* out /*
 
 /* Launch configuration chosen by igks_autotune. */
 typedef struct igks_tuning {
-  int32_t sweep_threads;   /* threads per block of the one-block-per-solve sweeps */
-  int32_t flux_block;      /* threads per block of the flux kernel */
+  int32_t sweep_threads;   /* cell threads of the sweeps (igks_options.sweep_threads): 128 or 256 */
+  int32_t flux_block;      /* threads per block of the flux kernel: 32 (untuned default), 64 or 128 */
   int32_t sweep_mode;      /* 1 one block per solve, 2 one launch per level */
   int32_t sweep_cluster;   /* blocks per solve of schedule 1 */
   float ms_per_iter;       /* measured device time of one iteration with it */

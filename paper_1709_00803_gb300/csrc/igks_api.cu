@@ -1342,7 +1342,7 @@ int igks_autotune(igks_ctx* ctx, int32_t iters_per_trial, igks_tuning* out) {
   igks_tuning best{};
   best.ms_per_iter = 1e30f;
   const bool wide_ok = std::max(d.n_wfwd, d.n_wbwd) <= 4 * WIDE_MAX_LEVELS;
-  const int flux_blocks[] = {64, 128};
+  const int flux_blocks[] = {32, 64, 128};   // (32: the untuned default)
   const int sweep_threads[] = {128, 256};
   const int clusters[] = {1, 2, 4};
   const int groups[] = {1, 2, 4, 8};
@@ -1395,7 +1395,7 @@ int igks_autotune(igks_ctx* ctx, int32_t iters_per_trial, igks_tuning* out) {
 
 int igks_set_launch(igks_ctx* ctx, const igks_tuning* t) {
   if (!ctx || !t) return IGKS_EINVAL;
-  if ((t->sweep_threads != 128 && t->sweep_threads != 256) || (t->flux_block != 64 && t->flux_block != 128) ||
+  if ((t->sweep_threads != 128 && t->sweep_threads != 256) || (t->flux_block != 32 && t->flux_block != 64 && t->flux_block != 128) ||
       (t->sweep_mode != 1 && t->sweep_mode != 2) ||
       (t->sweep_cluster != 1 && t->sweep_cluster != 2 && t->sweep_cluster != 4 && t->sweep_cluster != 8) ||
       t->groups < 1)
