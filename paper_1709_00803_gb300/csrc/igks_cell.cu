@@ -145,6 +145,7 @@ __device__ __forceinline__ long long ord_of(double x) {
   const long long b = __double_as_longlong(x);
   return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
+constexpr long long ORD_LOWEST = (long long)0x800fffffffffffffull;   // of minus infinity; negative NaNs are below it
 __device__ __forceinline__ double of_ord(long long k) {
   return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
 }
@@ -363,7 +364,8 @@ __global__ void __launch_bounds__(CELL_BLOCK * V) k_gradient(Dev d) {
             const double dp = __double2hiint(dv) < 0 ? lo[v] : hi[v];
             const double a = dp * dp, c = 2.0 * dv * dv;
             const double pv = ((a + eps2) * dv + c * dp) / (dv * (a + c + dv * dp + eps2));
-            if (ord_of(pv) < ord_of(phi[v])) phi[v] = pv;
+            const long long kp = ord_of(pv);   // (a quotient 0 / 0 of underflowed products is passed over)
+            if (kp < ord_of(phi[v]) && kp >= ORD_LOWEST) phi[v] = pv;
           }
         }
       }
