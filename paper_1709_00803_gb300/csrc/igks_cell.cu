@@ -479,7 +479,8 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_residual(Dev d) {
   }
   __shared__ double ssum[CELL_BLOCK / 32];
   __shared__ unsigned long long smax[CELL_BLOCK / 32];
-  const unsigned long long wm = warp_max(bits_of(rmax));
+  const unsigned long long rb = bits_of(rmax);        // (what is not a number does not count, as in fmax)
+  const unsigned long long wm = warp_max(rb > 0x7ff0000000000000ull ? 0ull : rb);
   for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
   if ((threadIdx.x & 31) == 0) { smax[threadIdx.x >> 5] = wm; ssum[threadIdx.x >> 5] = r2; }
   __syncthreads();
