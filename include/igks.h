@@ -84,7 +84,8 @@ typedef struct igks_options {
                              2 one launch per level over all solves (low-depth orderings) */
   int32_t sweep_cluster;  /* schedule 1: a thread-block cluster of 1 (0: 1), 2, 4 or 8 blocks per
                              solve shares each level (distributed shared memory, one cluster
-                             barrier per level); same arithmetic, same bits */
+                             barrier per level); with 1, solves of few broad levels (more than 512
+                             cells on average) have eight; same arithmetic, same bits */
   int32_t groups;         /* schedule 1 with several solves: split them into this many groups of
                              consecutive solves (0: 1), each iterated by a graph on a stream of
                              its own, so that one group's sweeps (one block per solve) overlap
@@ -251,7 +252,7 @@ typedef struct igks_tuning {
   int32_t sweep_threads;   /* cell threads of the sweeps (igks_options.sweep_threads): 128 or 256 */
   int32_t flux_block;      /* threads per block of the flux kernel: 32 (untuned default), 64 or 128 */
   int32_t sweep_mode;      /* 1 one block per solve, 2 one launch per level */
-  int32_t sweep_cluster;   /* blocks per solve of schedule 1 */
+  int32_t sweep_cluster;   /* blocks per solve of schedule 1 (igks_options.sweep_cluster) */
   float ms_per_iter;       /* measured device time of one iteration with it */
   int32_t groups;          /* groups of solves on streams of their own (igks_options.groups) */
 } igks_tuning;

@@ -282,6 +282,8 @@ static int capture_graphs(igks_ctx* ctx) {
   return 0;
 }
 
+static int broad_solve(const HostMesh& m) { return m.nc > (int64_t)BROAD_LEVEL * std::max(m.nlev_f, m.nlev_b); }
+
 // Split the solves into groups of consecutive solves with about equal cell counts (one
 // group with the wide schedule, whose per-level launches span all solves), give each its
 // launch ranges, a stream and timing events, and capture their graphs.
@@ -312,6 +314,8 @@ static int setup_groups(igks_ctx* ctx) {
     const int s0 = cut[g], s1 = cut[g + 1];
     v.g_solve0 = s0; v.g_nsolve = s1 - s0;
     v.sweeps = group_sweeps(ctx, s0, s1);
+    if (d.sweep_cluster == 1)
+      for (int s = s0; s < s1; s++) v.n_broad += broad_solve(ctx->meshes[s]);
     v.g_blk0 = ctx->cell_off[s0] / CELL_BLOCK;
     v.g_nblk = (s1 < ns ? ctx->cell_off[s1] : ctx->nc_pad) / CELL_BLOCK - v.g_blk0;
     v.g_face0 = ctx->face_off[s0];
@@ -674,6 +678,9 @@ static int build(igks_ctx* ctx) {
   UP(fj, fj); UP(bj, bj);
   UP(fside_ptr, fs.side_ptr); UP(fside_j, fs.side_j); UP(bside_ptr, bs.side_ptr); UP(bside_j, bs.side_j);
   UP(gent_ptr, gent_ptr); UP(gent_pos, gent_pos);
+  std::vector<int> broad(ns);
+  for (int s = 0; s < ns; s++) broad[s] = broad_solve(ctx->meshes[s]);
+  UP(broad, broad);
   d.ring = ring;
   AL(gprim, double, 6 * (size_t)nf);
   d.lgrad = (double*)d.sw_st;
@@ -1417,9 +1424,11 @@ int igks_launches_per_iteration(igks_ctx* ctx, int32_t* out) {
   if (!ctx || !out) return IGKS_EINVAL;
   int rc = build(ctx);
   if (rc) return rc;
-  const int sweeps = 1 + (ctx->dev.wide ? ctx->dev.n_wfwd + ctx->dev.n_wbwd : 2);
   *out = 0;
-  for (const Dev& d : ctx->gdev) *out += N_KERNEL_KINDS - 3 + (d.sweeps ? sweeps : 0);
+  for (const Dev& d : ctx->gdev) {
+    const int narrow = 2 * ((d.n_broad > 0) + (d.n_broad < d.g_nsolve));   // clusters, single blocks
+    *out += N_KERNEL_KINDS - 3 + (d.sweeps ? 1 + (d.wide ? d.n_wfwd + d.n_wbwd : narrow) : 0);
+  }
   return IGKS_OK;
 }
 

@@ -174,6 +174,9 @@ struct Dev {
   // wide schedule: cells of each level of all solves
   int wide;                      // 1: one launch per level; 0: one block per solve
   int sweep_cluster;             // narrow schedule: blocks (a thread-block cluster) per solve
+  const int* broad;              // [n_solves] levels of more than BROAD_LEVEL cells on average
+  int n_broad;                   // broad solves of the group that clusters sweep while one block each
+                                 // sweeps the others (0 with sweep_cluster > 1: all in clusters)
   const int* wfwd_cells; const int* wbwd_cells;
   const int* h_wfwd_ptr; const int* h_wbwd_ptr;   // HOST arrays of level offsets (launch sizes)
   int n_wfwd, n_wbwd;
@@ -250,6 +253,14 @@ constexpr int N_KERNEL_KINDS = 11;   // kernels of one iteration (the wide sweep
 constexpr int ring_slots(int t) { return t == 4 ? 2048 : 1024; }
 constexpr int SIDE = 32;             // side slots of a level (two sets, by the level's parity)
 constexpr int zero_slot(int t) { return ring_slots(t) + 2 * SIDE; }
+// Solves of few broad levels are swept by a cluster of blocks each, also where the others have one
+// block: what counts in a level is then the cells that work at once, not the time between two
+// barriers. Forward + backward, one block -> eight (one thread a cell in one block before): 10,000
+// multicoloured quads (two levels) FP32 234 + 241 -> 65 + 57 us (87 + 76), FP64 500 + 506 -> 96 + 90
+// (268 + 274); 6,504 polygons (levels of 650) double-float 496 + 524 -> 153 + 147 (348 + 375).
+// The line lies where one block lost to what it was before; levels of 250-500 cells are faster in
+// one block than then (490,000 quads as given, levels of 350: FP64 17.9 + 18.3 ms, 19.8 + 21.1).
+constexpr int BROAD_LEVEL = 512, BROAD_CLUSTER = 8;
 constexpr int NARROW_THREADS = 256;  // cell threads of the narrow sweeps at most (two per cell of a level)
 constexpr int DEFAULT_WAIT_LIMIT = 1 << 24;   // spins of a device wait (about a second)
 constexpr int MAX_BATCH_GRAPH_ITERS = 64;     // iterations captured in one whole-batch graph at most

@@ -1015,6 +1015,7 @@ __device__ __forceinline__ void sweep_narrow(const Dev& d) {
   const int s = d.g_solve0 + blockIdx.x / C, r = blockIdx.x % C;   // one cluster of C blocks per solve
   if (d.st[s].state != 0 || d.flow[s].scheme == 1) return;         // uniform over the cluster
   if (!FWD && d.tmo[s]) return;                                    // the forward sweep of this solve gave up
+  if (d.n_broad && (d.broad[s] != 0) != (C > 1)) return;           // the other launch sweeps it
   // (without SA its coefficients and 1/a_ii are zero and so are its increments: on the FP32
   // pipes the row is computed all the same, which costs less than the branches)
   const bool sa_on = std::is_same<T, double>::value ? d.flow[s].sa_on != 0 : true;
@@ -1281,6 +1282,8 @@ static void launch_cluster(const Dev& d, int threads, cudaStream_t s) {
 
 template <class T, bool FWD>
 static void launch_narrow(const Dev& d, int threads, cudaStream_t s) {
+  if (d.n_broad) launch_cluster<T, FWD, BROAD_CLUSTER>(d, threads, s);
+  if (d.n_broad == d.g_nsolve) return;
   switch (d.sweep_cluster) {
     case 2: launch_cluster<T, FWD, 2>(d, threads, s); break;
     case 4: launch_cluster<T, FWD, 4>(d, threads, s); break;

@@ -48,3 +48,27 @@ def test_shallow_mesh_beside_a_deep_one_bitwise(precision):
     deep = (G.plate_scaled(5003, 1), F.turbulent_plate_flow())
     for a, b in zip(_run([shallow, deep], precision), _run([shallow], precision, sweep_mode=2)):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("groups", [1, 2, 5])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_broad_and_thin_solves_in_one_context(precision, groups):
+    """Solves of few broad levels (clusters) between solves of many thin ones (a block each), in
+    groups that hold either kind or both: the bits of each solve alone, and the launches of each kind."""
+    from paper_1709_00803_gb300 import igks
+    broad = (MESHES["multicolour_plate"](), F.turbulent_plate_flow())
+    thin = (G.plate_scaled(2000, 1), F.turbulent_plate_flow())
+    solves = [broad, thin, thin, broad, broad]
+    alone = {id(s): _run([s], precision, iters=5)[2] for s in (broad, thin)}
+    ctx = igks.Context(precision=precision, groups=groups, check_every=2)
+    for m, fl in solves:
+        ctx.set_flow(ctx.mesh_upload(m), fl)
+    for k, (m, fl) in enumerate(solves):
+        ctx.init_freestream(k)
+        ctx.set_fields(k, F.perturbed_state(m, fl, seed=61, amp=0.02))
+    # nine kernels a group and two sweeps for each kind in it; of two groups the second is the last solve
+    assert ctx.launches_per_iteration() == {1: 13, 2: 13 + 11, 5: 5 * 11}[groups]
+    ctx.iterate(5)
+    for k, s in enumerate(solves):
+        assert np.array_equal(ctx.get_fields(k), alone[id(s)])
+    ctx.destroy()

@@ -30,6 +30,7 @@ def _rows_by_parity(nx, ny):
 
 MESHES = {
     "wide_then_thin": lambda: _half_multicolour(90, False),
+    "less_wide_then_thin": lambda: _half_multicolour(60, False),
     "thin_then_wide": lambda: _half_multicolour(90, True),
     "levels_of_500": lambda: _rows_by_parity(1000, 20),
     "levels_of_1000": lambda: _rows_by_parity(2000, 12),
@@ -63,6 +64,11 @@ def test_staged_levels_bitwise_and_starved_copy_noticed(name, precision):
     s = ctx.mesh_upload(m); ctx.set_flow(s, fl); ctx.init_freestream(s)
     ctx.set_fields(s, W0)
     rc, st = ctx.iterate(1)
+    info = ctx.mesh_info(s)
+    if m.n_cells > 512 * max(info["levels_fwd"], info["levels_bwd"]):   # in clusters: no copies to wait for
+        assert rc == igks.OK and name.startswith(("levels_of_500", "levels_of_1000", "two_levels"))
+        ctx.destroy()
+        return
     assert rc == igks.TIMEOUT and st[s]["state"] == igks.TIMEOUT
     assert np.array_equal(ctx.get_fields(s), W0)
     ctx.destroy()
