@@ -62,7 +62,7 @@ constexpr int SLOT_GLOBAL = -1, SLOT_GHOST = -2;
 constexpr int KIND_COUNT = 7;        // entries
 constexpr int KIND_THIRD = 8;        // a third entry, all three in ring or side slots
 constexpr int KIND_RARE = 16;        // a ghost, or a neighbour in global memory
-constexpr int KIND_SIDE = 32;        // a side slot (used by staged solves only)
+constexpr int KIND_SIDE = 32;        // a side slot (not in a cluster)
 constexpr int KIND_CSR = 64;         // more than PF_E entries: the CSR stencil (KIND_RARE too)
 constexpr int SPILL_READ = 1;        // a later cell reads this cell's increments from global memory
 constexpr int SPILL_OWN = 2;         // the level and the next do not fit the ring: no store warp takes it

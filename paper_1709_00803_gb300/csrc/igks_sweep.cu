@@ -546,10 +546,13 @@ __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int
 //    values are 48 or 96 bytes, which puts consecutive cells on distinct banks), SA apart.
 // Forward + backward on the 20,480-cell hybrid plate (351 levels each way), against one
 // thread per cell that read its record inside the level and stored its results itself:
-// FP32 401 + 418 -> 172 + 147 us, double-float 592 + 719 -> 344 + 316, FP64 1192 + 1417 ->
-// 756 + 695 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
+// FP32 401 + 418 -> 170 + 147 us, double-float 592 + 719 -> 340 + 318, FP64 1192 + 1417 ->
+// 746 + 684 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
 // 60,160-cell O-mesh (605 levels; every level has a seam cell whose neighbour left the ring
-// 300 levels ago) FP32 946 + 895 -> 442 + 444 us; 5,003 cells of plate 160 + 188 -> 61 + 58.
+// 300 levels ago) FP32 946 + 895 -> 442 + 446 us; 5,040 cells of plate 160 + 188 -> 60 + 59.
+// Every level counts by itself: where a deep solve has some levels wider than the record buffers
+// (250,368-cell O-mesh, 32 of 1,265 above 352 cells), double-float 5.85 + 6.31 -> 5.11 + 5.36 ms,
+// FP64 9.68 + 11.34 -> 8.52 + 8.76; staging none of such a solve's levels, 7.49 + 5.50 and 11.59 + 8.88.
 // A level ends when the store warps have stored the level before: one 16-byte store instead of
 // two of 8, and targets of two rounds read ahead instead of three, took FP32 forward from 184
 // and 492 to 176 and 457 us; a cell's increments side by side in dW (INC_STRIDE) took backward
