@@ -546,13 +546,13 @@ __device__ __forceinline__ void flush_eq40(const Dev& d, int s, double eq40, int
 //    values are 48 or 96 bytes, which puts consecutive cells on distinct banks), SA apart.
 // Forward + backward on the 20,480-cell hybrid plate (351 levels each way), against one
 // thread per cell that read its record inside the level and stored its results itself:
-// FP32 401 + 418 -> 170 + 147 us, double-float 592 + 719 -> 340 + 318, FP64 1192 + 1417 ->
-// 746 + 684 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
+// FP32 401 + 418 -> 169 + 149 us, double-float 592 + 719 -> 340 + 319, FP64 1192 + 1417 ->
+// 740 + 685 (FP64: 37 warp instructions a level at 64-76 cycles are most of it). The
 // 60,160-cell O-mesh (605 levels; every level has a seam cell whose neighbour left the ring
-// 300 levels ago) FP32 946 + 895 -> 442 + 446 us; 5,040 cells of plate 160 + 188 -> 60 + 59.
+// 300 levels ago) FP32 946 + 895 -> 439 + 450 us; 5,040 cells of plate 160 + 188 -> 59 + 59.
 // Every level counts by itself: where a deep solve has some levels wider than the record buffers
-// (250,368-cell O-mesh, 32 of 1,265 above 352 cells), double-float 5.85 + 6.31 -> 5.11 + 5.36 ms,
-// FP64 9.68 + 11.34 -> 8.52 + 8.76; staging none of such a solve's levels, 7.49 + 5.50 and 11.59 + 8.88.
+// (250,368-cell O-mesh, 32 of 1,265 above 352 cells), double-float 5.85 + 6.31 -> 5.03 + 5.37 ms,
+// FP64 9.68 + 11.34 -> 8.44 + 8.74; staging none of such a solve's levels, 7.49 + 5.50 and 11.59 + 8.88.
 // A level ends when the store warps have stored the level before: one 16-byte store instead of
 // two of 8, and targets of two rounds read ahead instead of three, took FP32 forward from 184
 // and 492 to 176 and 457 us; a cell's increments side by side in dW (INC_STRIDE) took backward
@@ -769,26 +769,26 @@ __device__ __forceinline__ void store_inc(const Dev& d, int at, const T* w, T w4
   }
 }
 
-// what a cell thread itself stores (before the barrier): the increments and flux increments that
-// a later cell reads from global memory (SPILL_READ), and the increments of a level that the
-// store warps do not take (SPILL_OWN; pb: the cell's backward position)
+// the increments of a cell that a later one reads from global memory (before the barrier)
 template <class T, bool FWD>
-__device__ __noinline__ void store_spill(const Dev& d, int i, int pb, int spill, LaneOut<T> o, int lane) {
+__device__ __noinline__ void store_spill(const Dev& d, int i, LaneOut<T> o, int lane) {
   const int n = d.nc_pad;
-  if (FWD && (spill & SPILL_OWN)) {
-    T* m = ((SweepRec<T>*)d.brec + pb)->m;
-    m[2 * lane] = o.w0;
-    m[2 * lane + 1] = o.w1;
-    if (lane) m[4] = o.w4;
-  }
-  if (FWD && !(spill & SPILL_READ)) return;
   T* dWv = (T*)(FWD ? d.dWs : d.dW);
   T* dF = (T*)d.dF;
   dWv[inc_at<T>(n, 2 * lane, i)] = o.w0;
   dWv[inc_at<T>(n, 2 * lane + 1, i)] = o.w1;
   if (lane) dWv[inc_at<T>(n, 4, i)] = o.w4;
-  if (!(spill & SPILL_READ)) return;
   for (int v = 0; v < 4; v++) dF[(2 * v + lane) * n + i] = o.f[v];
+}
+
+// the increments of a cell in a level that the store warps do not take (SPILL_OWN; at as in store_inc)
+template <class T, bool FWD>
+__device__ __noinline__ void store_own(const Dev& d, int at, LaneOut<T> o, int lane) {
+  const int n = d.nc_pad;
+  T* m = FWD ? ((SweepRec<T>*)d.brec + at)->m : (T*)d.dW;
+  m[FWD ? 2 * lane : inc_at<T>(n, 2 * lane, at)] = o.w0;
+  m[FWD ? 2 * lane + 1 : inc_at<T>(n, 2 * lane + 1, at)] = o.w1;
+  if (lane) m[FWD ? 4 : inc_at<T>(n, 4, at)] = o.w4;
 }
 
 // the accumulators of a cell with more entries than a record holds (p: its position)
@@ -917,8 +917,10 @@ __device__ __forceinline__ LaneOut<T> lane_cell(const Dev& d, T* ring, T* ring4,
   const LaneOut<T> o = lane_finish<T, FWD>(rc, acc0, acc1, acc4, lane, sa_on);
   if (valid) {
     ring_put<T>(ring + at.put, ring4 + at.put4, o, lane);
-    const int spill = C == 1 ? rc.spill : rc.spill & SPILL_READ;   // (a cluster's cells store all the same)
-    if (spill) store_spill<T, FWD>(d, rc.i, rc.pb, spill, o, lane);
+    if (rc.spill) {
+      if (C == 1 && (rc.spill & SPILL_OWN)) store_own<T, FWD>(d, FWD ? rc.pb : rc.i, o, lane);
+      if (rc.spill & SPILL_READ) store_spill<T, FWD>(d, rc.i, o, lane);
+    }
   }
   return o;
 }
